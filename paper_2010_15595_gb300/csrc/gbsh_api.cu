@@ -14,6 +14,7 @@
 #include "../../include/gbsh.h"
 #include "batch_host.h"
 #include "lhaf_kernels.cuh"
+#include "lhaf_tree.h"
 #include "tuning.h"
 
 namespace {
@@ -124,12 +125,36 @@ int run_sync(const gbsh::LhafPlan& plan, const double2* base, int ld, const doub
   return GBSH_OK;
 }
 
+// Whether a call that does not ask for sum |p_Z| is evaluated by the elimination tree
+// (lhaf_tree.cuh). The sum over |p_Z| only exists in the subset sum.
+bool tree_precision(int prec, int N) {
+  (void)N;
+  return prec == GBSH_PREC_TF;
+}
+
 double err_from(double abs_sum, gbsh_c128 v, int prec = GBSH_PREC_FP64) {
   double mag = std::hypot(v.re, v.im);
   if (mag == 0.0) return INFINITY;
   return unit_roundoff(prec) * abs_sum / mag;
 }
 
+// One evaluation by the elimination tree, its result copied to the host; *done = false when
+// the problem has to be evaluated by the subset sum.
+int tree_sync(gbsh::TreePlan* tp, const gbsh::BatchInput& in, void* ws, cudaStream_t st,
+              gbsh_c128* out, bool* done) {
+  GBSH_CUDA(gbsh::tree_stage(tp, &in, ws, st));
+  GBSH_CUDA(gbsh::tree_launch(*tp, ws, st));
+  double res[3];
+  GBSH_CUDA(cudaMemcpyAsync(res, static_cast<char*>(ws) + tp->off_out, sizeof(res),
+                            cudaMemcpyDeviceToHost, st));
+  GBSH_CUDA(cudaStreamSynchronize(st));
+  *done = res[2] == 0.0;
+  if (*done) {
+    out->re = res[0];
+    out->im = res[1];
+  }
+  return GBSH_OK;
+}
 
 // ---------------------------------------------------------------- batched evaluation
 using gbsh::BatchLayout;
@@ -149,40 +174,89 @@ bool valid_precision(int p) {
 }
 
 
-// Runs the batch in the requested precision. GBSH_PREC_MIXED evaluates the problems with
-// N <= GBSH_C32_MAX_N in complex FP32 and the others in FP64, as two launches that share
-// the workspace (the first `staged` bytes hold the caller's inputs).
-int batch_run_mixed(const int* Ns, const std::vector<gbsh::BatchInput>& in, int count,
-                    int precision, size_t staged, Scratch& s, void** ws, cudaStream_t st,
-                    double* out3) {
-  if (precision != GBSH_PREC_MIXED) {
-    BatchLayout L = batch_layout(Ns, count, staged);
-    int rc = scratch_get(s, L.bytes, ws);
-    if (rc != GBSH_OK) return rc;
-    return batch_run(L, in, count, precision, *ws, st, out3);
+// Runs the problems `sel` of a batch by the subset sum in `prec`, in the workspace behind the
+// first `staged` bytes (which hold the caller's inputs), and puts their results in place.
+int batch_run_some(const std::vector<int>& sel, const int* Ns, const std::vector<gbsh::BatchInput>& in,
+                   int prec, size_t staged, void* ws, cudaStream_t st, double* out3) {
+  if (sel.empty()) return GBSH_OK;
+  std::vector<int> Ns_sel(sel.size());
+  std::vector<gbsh::BatchInput> in_sel(sel.size());
+  for (size_t q = 0; q < sel.size(); ++q) {
+    Ns_sel[q] = Ns[sel[q]];
+    in_sel[q] = in[sel[q]];
   }
+  BatchLayout L = batch_layout(Ns_sel.data(), (int)sel.size(), staged);
+  std::vector<double> o((size_t)3 * sel.size());
+  int rc = batch_run(L, in_sel, (int)sel.size(), prec, ws, st, o.data());
+  if (rc != GBSH_OK) return rc;
+  for (size_t q = 0; q < sel.size(); ++q)
+    for (int j = 0; j < 3; ++j) out3[3 * (size_t)sel[q] + j] = o[3 * q + j];
+  return GBSH_OK;
+}
+
+// A batch's plan: its subset-sum layout (which bounds every part of the batch) and, when the
+// elimination tree evaluates it, the tree's.
+struct BatchPlan {
+  BatchLayout L;
+  bool tree = false;
+  std::vector<int> sel;  // problems of the tree (N > 0)
+  gbsh::TreePlan T;
+  size_t bytes = 0;
+};
+int batch_plan(const int* Ns, int count, int precision, bool want_abs, size_t staged, BatchPlan* B) {
+  B->L = batch_layout(Ns, count, staged);
+  B->bytes = B->L.bytes;
+  B->tree = !want_abs && precision == GBSH_PREC_TF;
+  if (!B->tree) return GBSH_OK;
+  std::vector<int> n;
+  for (int p = 0; p < count; ++p)
+    if (Ns[p] > 0) {
+      B->sel.push_back(p);
+      n.push_back(Ns[p]);
+    }
+  GBSH_CUDA(gbsh::tree_plan(n.data(), (int)n.size(), staged, &B->T));
+  B->bytes = std::max(B->bytes, B->T.bytes);
+  return GBSH_OK;
+}
+
+// Runs a planned batch in `precision`. GBSH_PREC_MIXED evaluates the problems with
+// N <= GBSH_C32_MAX_N in complex FP32 and the others in FP64, as two launches that share
+// the workspace. Problems that the tree hands back are evaluated by the subset sum.
+int batch_run_planned(BatchPlan* B, const int* Ns, const std::vector<gbsh::BatchInput>& in, int count,
+                      int precision, size_t staged, void* ws, cudaStream_t st, double* out3) {
+  if (B->tree) {
+    for (int p = 0; p < count; ++p)
+      if (Ns[p] == 0) {
+        out3[3 * (size_t)p] = 1.0;
+        out3[3 * (size_t)p + 1] = 0.0;
+        out3[3 * (size_t)p + 2] = 1.0;
+      }
+    std::vector<gbsh::BatchInput> in_sel(B->sel.size());
+    for (size_t q = 0; q < B->sel.size(); ++q) in_sel[q] = in[B->sel[q]];
+    std::vector<double> o((size_t)3 * B->sel.size());
+    GBSH_CUDA(gbsh::tree_stage(&B->T, in_sel.data(), ws, st));
+    GBSH_CUDA(gbsh::tree_launch(B->T, ws, st));
+    GBSH_CUDA(cudaMemcpyAsync(o.data(), static_cast<char*>(ws) + B->T.off_out, sizeof(double) * o.size(),
+                              cudaMemcpyDeviceToHost, st));
+    GBSH_CUDA(cudaStreamSynchronize(st));
+    std::vector<int> again;
+    for (size_t q = 0; q < B->sel.size(); ++q) {
+      const int p = B->sel[B->T.order[q]];
+      if (o[3 * q + 2] != 0.0) again.push_back(p);
+      out3[3 * (size_t)p] = o[3 * q];
+      out3[3 * (size_t)p + 1] = o[3 * q + 1];
+      out3[3 * (size_t)p + 2] = 0.0;
+    }
+    std::sort(again.begin(), again.end());
+    return batch_run_some(again, Ns, in, precision, staged, ws, st, out3);
+  }
+  if (precision != GBSH_PREC_MIXED) return batch_run(B->L, in, count, precision, ws, st, out3);
   for (int pass = 0; pass < 2; ++pass) {
-    const int prec = pass == 0 ? GBSH_PREC_C32 : GBSH_PREC_FP64;
     std::vector<int> sel;
     for (int p = 0; p < count; ++p)
       if ((Ns[p] <= GBSH_C32_MAX_N) == (pass == 0)) sel.push_back(p);
-    if (sel.empty()) continue;
-    std::vector<int> Ns_sel(sel.size());
-    std::vector<gbsh::BatchInput> in_sel(sel.size());
-    for (size_t q = 0; q < sel.size(); ++q) {
-      Ns_sel[q] = Ns[sel[q]];
-      in_sel[q] = in[sel[q]];
-    }
-    BatchLayout L = batch_layout(Ns_sel.data(), (int)sel.size(), staged);
-    void* before = *ws;
-    int rc = scratch_get(s, L.bytes, ws);
+    int rc = batch_run_some(sel, Ns, in, pass == 0 ? GBSH_PREC_C32 : GBSH_PREC_FP64, staged, ws, st, out3);
     if (rc != GBSH_OK) return rc;
-    if (*ws != before) return GBSH_ENOMEM;  // staged inputs must not move between passes
-    std::vector<double> o((size_t)3 * sel.size());
-    rc = batch_run(L, in_sel, (int)sel.size(), prec, *ws, st, o.data());
-    if (rc != GBSH_OK) return rc;
-    for (size_t q = 0; q < sel.size(); ++q)
-      for (int j = 0; j < 3; ++j) out3[3 * (size_t)sel[q] + j] = o[3 * q + j];
   }
   return GBSH_OK;
 }
@@ -238,7 +312,10 @@ size_t gbsh_lhaf_workspace_size_ex(int N, int precision) {
   if (N < 1 || N > GBSH_MAX_N) return 0;
   gbsh::LhafPlan plan;
   if (plan_for(N, &plan, precision) != GBSH_OK) return 0;
-  return plan.bytes;
+  if (!tree_precision(precision, N)) return plan.bytes;
+  gbsh::TreePlan tp;  // the tree's part follows the subset sum's: both stay usable in one call
+  if (gbsh::tree_plan(&N, 1, plan.bytes, &tp) != cudaSuccess) return 0;
+  return tp.bytes;
 }
 
 int gbsh_lhaf(const gbsh_c128* A, int N, int lda, gbsh_c128* out, double* err_est,
@@ -265,8 +342,14 @@ int gbsh_lhaf_ex(const gbsh_c128* A, int N, int lda, int precision, gbsh_c128* o
   Scratch& s = g_scratch[dev & 63];
   std::lock_guard<std::mutex> lk(s.mu);
   const bool on_dev = is_device_pointer(A);
+  const bool tree = !err_est && tree_precision(precision, N);
+  gbsh::TreePlan tp;
   const size_t in_off = align256(plan.bytes);
-  const size_t need = on_dev ? plan.bytes : in_off + sizeof(double2) * (size_t)N * N;
+  size_t need = on_dev ? plan.bytes : in_off + sizeof(double2) * (size_t)N * N;
+  if (tree) {
+    GBSH_CUDA(gbsh::tree_plan(&N, 1, need, &tp));
+    need = tp.bytes;
+  }
   void* ws = nullptr;
   rc = scratch_get(s, need, &ws);
   if (rc != GBSH_OK) return rc;
@@ -278,6 +361,11 @@ int gbsh_lhaf_ex(const gbsh_c128* A, int N, int lda, int precision, gbsh_c128* o
                                 sizeof(double2) * N, N, cudaMemcpyHostToDevice, st));
     base = dA;
     ld = N;
+  }
+  if (tree) {
+    bool done = false;
+    rc = tree_sync(&tp, gbsh::BatchInput{base, nullptr, nullptr, ld, N}, ws, st, out, &done);
+    if (rc != GBSH_OK || done) return rc;
   }
   double asum = 0.0;
   rc = run_sync(plan, base, ld, nullptr, nullptr, ws, st, out, &asum);
@@ -307,6 +395,23 @@ int gbsh_lhaf_async_ex(const gbsh_c128* dA, int N, int lda, int precision, gbsh_
   int rc = plan_for(N, &plan, precision);
   if (rc != GBSH_OK) return rc;
   if (workspace_bytes < plan.bytes) return GBSH_EINVAL;
+  bool tree = !d_abs_sum && tree_precision(precision, N);
+  gbsh::TreePlan tp;
+  if (tree) {
+    GBSH_CUDA(gbsh::tree_plan(&N, 1, plan.bytes, &tp));
+    tree = workspace_bytes >= tp.bytes;
+  }
+  if (tree) {
+    // The tree writes the result; the subset sum follows, gated by the tree's flag, and its
+    // kernels return at once unless the problem has to be evaluated that way.
+    double* value = reinterpret_cast<double*>(d_out);
+    const gbsh::BatchInput in{reinterpret_cast<const double2*>(dA), nullptr, nullptr, lda, N};
+    GBSH_CUDA(gbsh::tree_stage(&tp, &in, workspace, st));
+    GBSH_CUDA(gbsh::tree_launch(tp, workspace, st, value));
+    GBSH_CUDA(gbsh::launch_range(plan, in.base, lda, nullptr, nullptr, workspace, st, 0,
+                                 (uint64_t)1 << plan.n, gbsh::tree_flag(tp, workspace), value));
+    return GBSH_OK;
+  }
   GBSH_CUDA(gbsh::launch_lhaf(plan, reinterpret_cast<const double2*>(dA), lda, nullptr,
                               nullptr, workspace, st));
   const char* res = static_cast<const char*>(workspace) + plan.off_out;
@@ -477,9 +582,11 @@ int gbsh_lhaf_batch(const gbsh_c128* A_packed, const int64_t* offsets, const int
   std::lock_guard<std::mutex> lk(s.mu);
   const bool on_dev = is_device_pointer(A_packed);
   const size_t in_bytes = on_dev ? 0 : sizeof(double2) * (size_t)span;
-  BatchLayout L = batch_layout(Ns, count, in_bytes);
+  BatchPlan B;
+  int rc = batch_plan(Ns, count, precision, abs_sums != nullptr, in_bytes, &B);
+  if (rc != GBSH_OK) return rc;
   void* ws = nullptr;
-  int rc = scratch_get(s, L.bytes, &ws);  // the full layout bounds every sub-batch
+  rc = scratch_get(s, B.bytes, &ws);
   if (rc != GBSH_OK) return rc;
   const double2* base = reinterpret_cast<const double2*>(A_packed);
   if (!on_dev) {
@@ -489,7 +596,7 @@ int gbsh_lhaf_batch(const gbsh_c128* A_packed, const int64_t* offsets, const int
   std::vector<gbsh::BatchInput> in(count);
   for (int p = 0; p < count; ++p) in[p] = gbsh::BatchInput{base + offsets[p], nullptr, nullptr, Ns[p], Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_mixed(Ns, in, count, precision, in_bytes, s, &ws, st, out3.data());
+  rc = batch_run_planned(&B, Ns, in, count, precision, in_bytes, ws, st, out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     outs[p].re = out3[3 * p];
@@ -539,9 +646,12 @@ int gbsh_gbs_prob_batch(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gam
   const size_t idx_bytes = align256(sizeof(int) * std::max<size_t>(idx.size(), 1));
   const size_t b_bytes = on_dev ? 0 : align256(sizeof(double2) * (size_t)M * M);
   const size_t g_bytes = on_dev ? 0 : align256(sizeof(double2) * (size_t)g_elems);
-  BatchLayout L = batch_layout(Ns.data(), count, idx_bytes + b_bytes + g_bytes);
+  const size_t staged = idx_bytes + b_bytes + g_bytes;
+  BatchPlan plan;
+  int rc = batch_plan(Ns.data(), count, precision, false, staged, &plan);
+  if (rc != GBSH_OK) return rc;
   void* ws = nullptr;
-  int rc = scratch_get(s, L.bytes, &ws);
+  rc = scratch_get(s, plan.bytes, &ws);
   if (rc != GBSH_OK) return rc;
   char* w = static_cast<char*>(ws);
   int* d_idx = reinterpret_cast<int*>(w);
@@ -565,8 +675,7 @@ int gbsh_gbs_prob_batch(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gam
   for (int p = 0; p < count; ++p)
     in[p] = gbsh::BatchInput{dB, dg + gstride * p, d_idx + idx_off[p], ld, Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_mixed(Ns.data(), in, count, precision, idx_bytes + b_bytes + g_bytes, s, &ws, st,
-                       out3.data());
+  rc = batch_run_planned(&plan, Ns.data(), in, count, precision, staged, ws, st, out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     const double re = out3[3 * p], im = out3[3 * p + 1];

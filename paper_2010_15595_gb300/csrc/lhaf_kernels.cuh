@@ -61,9 +61,12 @@ cudaError_t launch_lhaf(const LhafPlan& plan, const double2* base, int ld, const
 
 // launch_lhaf restricted to the enumeration indices [i_begin, i_end) (expansion from `base`,
 // `diag`, `idx` as in launch_lhaf); the range's compensated partial as for launch_lhaf_range.
+// gate: device flag or null; where it is 0 when the kernels run, they find nothing to do and
+// write no result (the fallback of an evaluation whose caller cannot wait for the flag).
+// value: device pointer or null, receives the sum (re, im).
 cudaError_t launch_range(const LhafPlan& plan, const double2* base, int ld, const double2* diag,
                          const int* idx, void* ws, cudaStream_t stream, uint64_t i_begin,
-                         uint64_t i_end);
+                         uint64_t i_end, const unsigned* gate = nullptr, double* value = nullptr);
 
 // The subsets of the enumeration indices [i_begin, i_end) only (z = i ^ (i >> 1); any
 // partition of [0, 2^n) into such ranges covers every subset once). Writes the range's

@@ -1,0 +1,63 @@
+// Host interface of the elimination-tree evaluation (lhaf_tree.cu; the method is described in
+// lhaf_tree.cuh).
+#pragma once
+
+#include <cstddef>
+#include <vector>
+
+#include <cuda_runtime.h>
+
+#include "lhaf_types.cuh"
+
+namespace gbsh {
+
+// One problem of a launch. Its levels n .. m1 are computed breadth first by the whole GPU; each
+// node of level m1 is a unit that one CTA works off: depth first, two nodes a level, down to
+// level `top`, then breadth first.
+struct TreeProblem {
+  BatchInput in;
+  int Ne, n;       // padded size, Ne = 2 n >= 4
+  int m1, top;
+  unsigned unit_base, units;
+  size_t root;     // element offset of its levels n .. m1
+};
+
+// Running state of a problem: exact limb sums of the signed mean, and how to undo the scale.
+struct TreeState {
+  unsigned long long sum[6];
+  double fac_hi, fac_lo;
+  int exp2;
+  unsigned done;
+  unsigned bad;    // overflow, or a result too small for the fixed-point resolution
+  unsigned pad;
+};
+
+// Layout of the evaluation of `count` problems in one workspace (byte offsets).
+struct TreePlan {
+  std::vector<TreeProblem> prob;   // in launch order
+  std::vector<int> order;          // prob[q] is the caller's problem order[q]
+  unsigned total_units;
+  int blocks;
+  struct Step { int problems; unsigned tasks; };
+  std::vector<Step> steps;         // breadth-first eliminations: problems that take part (the
+                                   // first ones), most tasks of one of them
+  size_t cta_elems;                // scratch elements per CTA
+  size_t off_prob, off_state, off_counter, off_out, off_root, off_cta, bytes;
+};
+
+// Sizes 0 are left out (their loop hafnian is 1): `Ns` entries must be 1..kMaxN.
+cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan);
+
+// Evaluates the problems of `plan` (in[i]: input of the caller's problem i) in `ws` on `st`.
+// Result of launch-order problem q: three doubles at off_out + 24 q: re, im, and 1 where the
+// problem has to be evaluated by the subset sum instead (0 otherwise). `value` (one-problem
+// launches): device pointer that receives re, im instead; the flag is then at tree_flag().
+cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* value = nullptr);
+
+// Fills in the inputs and, for more than one problem, uploads the table.
+cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st);
+
+// Device address of a one-problem launch's fallback flag (nonzero: evaluate by the subset sum).
+const unsigned* tree_flag(const TreePlan& plan, void* ws);
+
+}  // namespace gbsh

@@ -184,14 +184,15 @@ def lhaf(A, stream=None, return_error=False, precision=None):
     ptr, N, ld, keep = _as_matrix(A)
     out = C128()
     err = ctypes.c_double()
+    perr = ctypes.byref(err) if return_error else None  # the estimate needs the subset sum
     st = ctypes.c_void_p(_stream_handle(stream))
     if precision is None:
         rc = load().gbsh_lhaf(ctypes.c_void_p(ptr if N else 0), N, max(ld, N), ctypes.byref(out),
-                              ctypes.byref(err), st)
+                              perr, st)
         _check(rc, "gbsh_lhaf")
     else:
         rc = load().gbsh_lhaf_ex(ctypes.c_void_p(ptr if N else 0), N, max(ld, N), int(precision),
-                                 ctypes.byref(out), ctypes.byref(err), st)
+                                 ctypes.byref(out), perr, st)
         _check(rc, "gbsh_lhaf_ex")
     val = complex(out.re, out.im)
     return (val, err.value) if return_error else val
@@ -370,7 +371,8 @@ def lhaf_batch(mats, precision=PREC_FP64, stream=None, return_abs_sum=False):
     sums = np.zeros(len(mats), dtype=np.float64)
     rc = load().gbsh_lhaf_batch(ctypes.c_void_p(packed.ctypes.data), ctypes.c_void_p(offs.ctypes.data),
                                 ctypes.c_void_p(Ns.ctypes.data), len(mats),
-                                ctypes.c_void_p(outs.ctypes.data), ctypes.c_void_p(sums.ctypes.data),
+                                ctypes.c_void_p(outs.ctypes.data),
+                                ctypes.c_void_p(sums.ctypes.data if return_abs_sum else 0),
                                 int(precision), ctypes.c_void_p(_stream_handle(stream)))
     _check(rc, "gbsh_lhaf_batch")
     return (outs, sums) if return_abs_sum else outs
