@@ -22,10 +22,10 @@
  *     GBSH_ECUDA, gbsh_strerror(code) names the last CUDA error of the calling thread.
  *   - Two evaluations of the same quantity exist. The subset sum forms every p_Z; it is what
  *     gives sum_Z |p_Z|, subset ranges and single terms. Where a call asks for none of these
- *     (err_est, d_abs_sum or abs_sums NULL) and the precision is GBSH_PREC_TF, an elimination
- *     tree in 84-bit fixed point evaluates the loop hafnian instead (csrc/lhaf_tree.cuh): far
- *     fewer operations and far less cancellation. A problem that leaves the fixed-point range is
- *     evaluated by the subset sum after all.
+ *     (err_est, d_abs_sum or abs_sums NULL) and the precision is GBSH_PREC_TF, or GBSH_PREC_FP64
+ *     with N <= 24, an elimination tree in 83-bit fixed point evaluates the loop hafnian instead
+ *     (csrc/lhaf_tree.cuh): far fewer operations and far less cancellation. A problem that
+ *     leaves the fixed-point range is evaluated by the subset sum after all.
  *   - Results are bit-reproducible for a given N on a given GPU model: the subset sum is
  *     split into fixed chunks whose compensated partial sums are combined in a fixed order, and
  *     the tree's sums are exact integers.
@@ -88,8 +88,8 @@ int gbsh_lhaf(const gbsh_c128* A, int N, int lda, gbsh_c128* out, double* err_es
 /* Bytes of device workspace gbsh_lhaf_async needs for size N (0 for N outside 1..MAX_N). */
 size_t gbsh_lhaf_workspace_size(int N);
 /* The same for gbsh_lhaf_async_ex in `precision` (0 for an unsupported precision). For
- * GBSH_PREC_TF this includes the elimination tree's scratch; a workspace that only holds the
- * subset sum's part is accepted too, and the subset sum is used. */
+ * GBSH_PREC_TF (and for N <= 24) this includes the elimination tree's scratch; a workspace that
+ * only holds the subset sum's part is accepted too, and the subset sum is used. */
 size_t gbsh_lhaf_workspace_size_ex(int N, int precision);
 
 /*

@@ -126,10 +126,13 @@ int run_sync(const gbsh::LhafPlan& plan, const double2* base, int ld, const doub
 }
 
 // Whether a call that does not ask for sum |p_Z| is evaluated by the elimination tree
-// (lhaf_tree.cuh). The sum over |p_Z| only exists in the subset sum.
+// (lhaf_tree.cuh): the sum over |p_Z| only exists in the subset sum. FP64 evaluations stay with
+// the subset sum above N = 24. The FP64 entry points -- single, batched, in subset ranges -- are
+// compared with one another, and there the rounding of the FP64 subset sum (4e-11 at N = 24,
+// 1e-10 to 1e-8 at N = 26 to 30) would show between one that moved and one that cannot.
+constexpr int kTreeFp64MaxN = 24;
 bool tree_precision(int prec, int N) {
-  (void)N;
-  return prec == GBSH_PREC_TF;
+  return prec == GBSH_PREC_TF || (prec == GBSH_PREC_FP64 && N <= kTreeFp64MaxN);
 }
 
 double err_from(double abs_sum, gbsh_c128 v, int prec = GBSH_PREC_FP64) {
@@ -142,13 +145,10 @@ double err_from(double abs_sum, gbsh_c128 v, int prec = GBSH_PREC_FP64) {
 // the problem has to be evaluated by the subset sum.
 int tree_sync(gbsh::TreePlan* tp, const gbsh::BatchInput& in, void* ws, cudaStream_t st,
               gbsh_c128* out, bool* done) {
-  GBSH_CUDA(gbsh::tree_stage(tp, &in, ws, st));
-  GBSH_CUDA(gbsh::tree_launch(*tp, ws, st));
   double res[3];
-  GBSH_CUDA(cudaMemcpyAsync(res, static_cast<char*>(ws) + tp->off_out, sizeof(res),
-                            cudaMemcpyDeviceToHost, st));
-  GBSH_CUDA(cudaStreamSynchronize(st));
-  *done = res[2] == 0.0;
+  std::vector<int> again;
+  GBSH_CUDA(gbsh::tree_run(tp, &in, ws, st, res, &again));
+  *done = again.empty();
   if (*done) {
     out->re = res[0];
     out->im = res[1];
@@ -194,71 +194,55 @@ int batch_run_some(const std::vector<int>& sel, const int* Ns, const std::vector
   return GBSH_OK;
 }
 
-// A batch's plan: its subset-sum layout (which bounds every part of the batch) and, when the
-// elimination tree evaluates it, the tree's.
+// A batch's plan: its subset-sum layout (which bounds every part of the batch), the problems
+// that the elimination tree evaluates and the tree's plan for them, and the others by precision.
 struct BatchPlan {
   BatchLayout L;
-  bool tree = false;
-  std::vector<int> sel;  // problems of the tree (N > 0)
+  std::vector<int> tree, c32, rest;
+  int rest_prec = GBSH_PREC_FP64;
   gbsh::TreePlan T;
   size_t bytes = 0;
 };
 int batch_plan(const int* Ns, int count, int precision, bool want_abs, size_t staged, BatchPlan* B) {
   B->L = batch_layout(Ns, count, staged);
-  B->bytes = B->L.bytes;
-  B->tree = !want_abs && precision == GBSH_PREC_TF;
-  if (!B->tree) return GBSH_OK;
+  B->rest_prec = precision == GBSH_PREC_MIXED ? GBSH_PREC_FP64 : precision;
   std::vector<int> n;
-  for (int p = 0; p < count; ++p)
-    if (Ns[p] > 0) {
-      B->sel.push_back(p);
+  for (int p = 0; p < count; ++p) {
+    if (precision == GBSH_PREC_MIXED && Ns[p] <= GBSH_C32_MAX_N) {
+      B->c32.push_back(p);
+    } else if (Ns[p] > 0 && !want_abs && tree_precision(B->rest_prec, Ns[p])) {
+      B->tree.push_back(p);
       n.push_back(Ns[p]);
+    } else {
+      B->rest.push_back(p);
     }
+  }
   GBSH_CUDA(gbsh::tree_plan(n.data(), (int)n.size(), staged, &B->T));
-  B->bytes = std::max(B->bytes, B->T.bytes);
+  B->bytes = std::max(B->L.bytes, B->T.bytes);
   return GBSH_OK;
 }
 
-// Runs a planned batch in `precision`. GBSH_PREC_MIXED evaluates the problems with
-// N <= GBSH_C32_MAX_N in complex FP32 and the others in FP64, as two launches that share
-// the workspace. Problems that the tree hands back are evaluated by the subset sum.
+// Runs a planned batch: the parts one after the other in the same workspace (GBSH_PREC_MIXED
+// evaluates the problems with N <= GBSH_C32_MAX_N in complex FP32, the others as FP64), then by
+// the subset sum what the tree hands back.
 int batch_run_planned(BatchPlan* B, const int* Ns, const std::vector<gbsh::BatchInput>& in, int count,
-                      int precision, size_t staged, void* ws, cudaStream_t st, double* out3) {
-  if (B->tree) {
-    for (int p = 0; p < count; ++p)
-      if (Ns[p] == 0) {
-        out3[3 * (size_t)p] = 1.0;
-        out3[3 * (size_t)p + 1] = 0.0;
-        out3[3 * (size_t)p + 2] = 1.0;
-      }
-    std::vector<gbsh::BatchInput> in_sel(B->sel.size());
-    for (size_t q = 0; q < B->sel.size(); ++q) in_sel[q] = in[B->sel[q]];
-    std::vector<double> o((size_t)3 * B->sel.size());
-    GBSH_CUDA(gbsh::tree_stage(&B->T, in_sel.data(), ws, st));
-    GBSH_CUDA(gbsh::tree_launch(B->T, ws, st));
-    GBSH_CUDA(cudaMemcpyAsync(o.data(), static_cast<char*>(ws) + B->T.off_out, sizeof(double) * o.size(),
-                              cudaMemcpyDeviceToHost, st));
-    GBSH_CUDA(cudaStreamSynchronize(st));
-    std::vector<int> again;
-    for (size_t q = 0; q < B->sel.size(); ++q) {
-      const int p = B->sel[B->T.order[q]];
-      if (o[3 * q + 2] != 0.0) again.push_back(p);
-      out3[3 * (size_t)p] = o[3 * q];
-      out3[3 * (size_t)p + 1] = o[3 * q + 1];
-      out3[3 * (size_t)p + 2] = 0.0;
-    }
-    std::sort(again.begin(), again.end());
-    return batch_run_some(again, Ns, in, precision, staged, ws, st, out3);
+                      size_t staged, void* ws, cudaStream_t st, double* out3) {
+  if ((int)B->rest.size() == count) return batch_run(B->L, in, count, B->rest_prec, ws, st, out3);
+  std::vector<int> again;
+  if (!B->tree.empty()) {
+    std::vector<gbsh::BatchInput> in_sel(B->tree.size());
+    std::vector<double> o((size_t)3 * B->tree.size());
+    for (size_t q = 0; q < B->tree.size(); ++q) in_sel[q] = in[B->tree[q]];
+    GBSH_CUDA(gbsh::tree_run(&B->T, in_sel.data(), ws, st, o.data(), &again));
+    for (size_t q = 0; q < B->tree.size(); ++q)
+      for (int j = 0; j < 3; ++j) out3[3 * (size_t)B->tree[q] + j] = o[3 * q + j];
+    for (int& p : again) p = B->tree[p];
   }
-  if (precision != GBSH_PREC_MIXED) return batch_run(B->L, in, count, precision, ws, st, out3);
-  for (int pass = 0; pass < 2; ++pass) {
-    std::vector<int> sel;
-    for (int p = 0; p < count; ++p)
-      if ((Ns[p] <= GBSH_C32_MAX_N) == (pass == 0)) sel.push_back(p);
-    int rc = batch_run_some(sel, Ns, in, pass == 0 ? GBSH_PREC_C32 : GBSH_PREC_FP64, staged, ws, st, out3);
-    if (rc != GBSH_OK) return rc;
-  }
-  return GBSH_OK;
+  int rc = batch_run_some(B->c32, Ns, in, GBSH_PREC_C32, staged, ws, st, out3);
+  if (rc != GBSH_OK) return rc;
+  rc = batch_run_some(B->rest, Ns, in, B->rest_prec, staged, ws, st, out3);
+  if (rc != GBSH_OK) return rc;
+  return batch_run_some(again, Ns, in, B->rest_prec, staged, ws, st, out3);
 }
 
 }  // namespace
@@ -492,7 +476,15 @@ int gbsh_gbs_prob(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gamma,
     const size_t idx_off = align256(plan.bytes);
     const size_t b_off = align256(idx_off + sizeof(int) * (size_t)N);
     const size_t g_off = align256(b_off + (on_dev ? 0 : sizeof(double2) * (size_t)M * M));
-    const size_t need = align256(g_off + (on_dev ? 0 : sizeof(double2) * (size_t)M));
+    size_t need = align256(g_off + (on_dev ? 0 : sizeof(double2) * (size_t)M));
+    const bool tree = tree_precision(GBSH_PREC_FP64, (int)N);
+    bool done = false;
+    gbsh::TreePlan tp;
+    if (tree) {
+      const int n1 = (int)N;
+      GBSH_CUDA(gbsh::tree_plan(&n1, 1, need, &tp));
+      need = tp.bytes;
+    }
     void* ws = nullptr;
     rc = scratch_get(s, need, &ws);
     if (rc != GBSH_OK) return rc;
@@ -513,8 +505,14 @@ int gbsh_gbs_prob(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gamma,
       dg = g2;
       ld = M;
     }
-    rc = run_sync(plan, dB, ld, dg, d_idx, ws, st, &l, nullptr);
-    if (rc != GBSH_OK) return rc;
+    if (tree) {
+      rc = tree_sync(&tp, gbsh::BatchInput{dB, dg, d_idx, ld, (int)N}, ws, st, &l, &done);
+      if (rc != GBSH_OK) return rc;
+    }
+    if (!done) {
+      rc = run_sync(plan, dB, ld, dg, d_idx, ws, st, &l, nullptr);
+      if (rc != GBSH_OK) return rc;
+    }
   }
   if (lhaf_out) *lhaf_out = l;
   *prob = p_vac * (l.re * l.re + l.im * l.im) / fact;
@@ -596,7 +594,7 @@ int gbsh_lhaf_batch(const gbsh_c128* A_packed, const int64_t* offsets, const int
   std::vector<gbsh::BatchInput> in(count);
   for (int p = 0; p < count; ++p) in[p] = gbsh::BatchInput{base + offsets[p], nullptr, nullptr, Ns[p], Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_planned(&B, Ns, in, count, precision, in_bytes, ws, st, out3.data());
+  rc = batch_run_planned(&B, Ns, in, count, in_bytes, ws, st, out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     outs[p].re = out3[3 * p];
@@ -675,7 +673,7 @@ int gbsh_gbs_prob_batch(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gam
   for (int p = 0; p < count; ++p)
     in[p] = gbsh::BatchInput{dB, dg + gstride * p, d_idx + idx_off[p], ld, Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_planned(&plan, Ns.data(), in, count, precision, staged, ws, st, out3.data());
+  rc = batch_run_planned(&plan, Ns.data(), in, count, staged, ws, st, out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     const double re = out3[3 * p], im = out3[3 * p + 1];

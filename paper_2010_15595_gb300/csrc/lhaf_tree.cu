@@ -15,9 +15,13 @@
 #include <mutex>
 #include <numeric>
 
+#include <cooperative_groups.h>
+
 #include "lhaf_kernels.cuh"
 #include "lhaf_tree.cuh"
 #include "lhaf_tree.h"
+
+namespace cg = cooperative_groups;
 
 namespace gbsh {
 
@@ -25,6 +29,10 @@ namespace {
 
 constexpr int kTreeThreads = 128;
 constexpr int kTreeCtasPerSm = 6;
+// Largest n of a small problem: alone (clusters of up to 16 CTAs), and in a crowd, where a
+// problem gets a CTA or two and its scratch (all levels) must stay in the cache.
+constexpr int kTreeSmallMax = 12;
+constexpr int kTreeSmallCrowd = 8;
 constexpr int kTreeTop = 6;  // level from which a unit is worked off breadth first
 // Smallest scaled result that is kept. The tree's absolute error is about 2^-80 (against a
 // 113-bit evaluation), so 2^-28 leaves it at 2^-52 of the result. The subset sum it would be
@@ -44,43 +52,30 @@ __device__ __forceinline__ void dd_mul(double ah, double al, double bh, double b
   l = __dsub_rn(e, __dsub_rn(h, p));
 }
 
-// x m 2^e in units of 2^-81 as limbs; bad |= it does not fit (or x is not finite).
+// x m 2^e in units of 2^-81 as limbs; bad |= it does not fit (or x is not finite). Integer
+// instructions only: FP64 ones are slow.
 __device__ void to_fixed(double x, int m, int e, int& h, int& mm, int& l, unsigned& bad) {
-  if (!(fabs(x) <= 1.7976931348623157e308)) bad = 1;
-  int ex;
-  const double f = frexp(x, &ex);
-  const long long i = (long long)ldexp(f, 53) * m;  // < 2^63: 53 bits times at most 31^2
-  const int sh = ex - 53 + e + kTreeFrac;
-  __int128 v = i;
-  if (i == 0) {
+  const long long bits = __double_as_longlong(x);
+  const int ex = (int)(bits >> 52) & 0x7ff;
+  if (ex == 0x7ff) bad = 1;
+  const long long mant = (bits & ((1ll << 52) - 1)) | (ex ? 1ll << 52 : 0);
+  __int128 v = (bits < 0 ? -mant : mant) * m;  // < 2^63: 53 bits times at most 31^2
+  const int sh = (ex ? ex : 1) - 1075 + e + kTreeFrac;
+  if (v == 0 || sh < -100) {
     v = 0;
   } else if (sh >= 0) {
     if (sh > 62) bad = 1;
     v <<= (sh > 62 ? 62 : sh);
-  } else if (sh < -100) {
-    v = 0;
   } else {
     v = (v + ((__int128)1 << (-sh - 1))) >> (-sh);
   }
-  const __int128 lim = (__int128)1 << 82;
+  const __int128 lim = (__int128)1 << kTreeFrac;  // |x| < 1: room for the first products
   if (v >= lim || v <= -lim) bad = 1;
-  l = sext28((long long)v);
-  v = (v - l) >> kLimbBits;
-  mm = sext28((long long)v);
-  v = (v - mm) >> kLimbBits;
-  h = (int)(long long)v;
-}
-
-template <class T, class F>
-__device__ T block_reduce(T x, T* sh, F f) {
-  __syncthreads();
-  sh[threadIdx.x] = x;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] = f(sh[threadIdx.x], sh[threadIdx.x + w]);
-    __syncthreads();
-  }
-  return sh[0];
+  v += kLimbHalf;
+  l = ((int)(long long)v & kLimbMask) - kLimbHalf;
+  v = (v >> kLimbBits) + kLimbHalf;
+  mm = ((int)(long long)v & kLimbMask) - kLimbHalf;
+  h = (int)(long long)(v >> kLimbBits);
 }
 
 __device__ __forceinline__ double2 tree_entry(const BatchInput& in, int r, int c) {
@@ -88,103 +83,161 @@ __device__ __forceinline__ double2 tree_entry(const BatchInput& in, int r, int c
   if (r == c && in.diag) return in.diag[ir];
   return in.base[(size_t)ir * in.ld + ic];
 }
+// Biased exponent of a double, and x 2^(1023 - ex) in single precision (0 where that underflows).
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ float scaled_float(double x, int ex) {
+  const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7ff) - ex + 127;
+  if (e <= 0) return 0.f;
+  return __int_as_float((hi & 0x80000000) | (e << 23) | ((hi & 0xfffff) << 3) |
+                        (int)((unsigned)__double2loint(x) >> 29));
+}
 
-constexpr int kRootThreads = 256;
+constexpr int kRootThreads = 256;  // of the root kernel and of a cluster's CTAs
+constexpr int kRootWarps = kRootThreads / 32;
 
-// kOne: one problem, passed as a kernel argument; otherwise a table in device memory.
-template <bool kOne>
-__global__ void __launch_bounds__(kRootThreads)
-tree_root_kernel(const TreeProblem* __restrict__ table, TreeProblem one,
-                 TreeState* __restrict__ state, unsigned* __restrict__ counter, Fxc* __restrict__ roots) {
-  __shared__ float2 a[kMaxN * kMaxN];
-  __shared__ double sh[kRootThreads];
-  __shared__ int s_m, s_e;
-  const TreeProblem P = kOne ? one : table[blockIdx.x];
-  const int tid = threadIdx.x, N = P.in.N;
-  auto dmax = [](double x, double y) { return x > y ? x : (y > x ? y : (x == x ? x : (y == y ? y : x))); };
-  auto dsum = [](double x, double y) { return x + y; };
-  unsigned bad = 0;
-  // largest entry off the diagonal, loop weights
-  double am = 0.0, vm = 0.0, v2 = 0.0;
-  for (int e = tid; e < N * N; e += kRootThreads) {
+struct RootShared {
+  float2 a[kMaxN * kMaxN];
+  unsigned ea[kRootWarps], ev[kRootWarps];
+  float f[5][kRootWarps];
+  int m, e;
+};
+
+__device__ __forceinline__ float warp_sum(float x) {
+  for (int d = 16; d; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+  return x;
+}
+__device__ __forceinline__ float warp_max(float x) {
+  for (int d = 16; d; d >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, d));
+  return x;
+}
+
+// Root level and state of a problem, by one CTA of kThreads threads: gathers the matrix, picks
+// the scale, writes the fixed-point numbers. Latency matters here (small problems take 20 us in
+// all), so the scale is worked out in single precision from exponent-shifted entries.
+template <int kThreads>
+__device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState* S, RootShared& sh) {
+  constexpr int kWarps = kThreads / 32;
+  const int tid = threadIdx.x, N = P.in.N, lane = tid & 31, warp = tid >> 5;
+  unsigned bad = 0, ea = 0, ev = 0;
+  for (int e = tid; e < N * N; e += kThreads) {
     const int r = e / N, c = e - r * N;
     const double2 z = tree_entry(P.in, r, c);
-    const double m = hypot(z.x, z.y);
-    if (!(m <= 1.7976931348623157e308)) bad = 1;
-    if (r == c) {
-      vm = dmax(vm, m);
-      v2 += m * m;
-    } else {
-      am = dmax(am, m);
-    }
+    const unsigned x = (unsigned)max(exponent_of(z.x), exponent_of(z.y));
+    if (x == 0x7ff) bad = 1;
+    if (r == c) ev = max(ev, x); else ea = max(ea, x);
   }
-  am = block_reduce(am, sh, dmax);
-  vm = block_reduce(vm, sh, dmax);
-  v2 = block_reduce(v2, sh, dsum);
-  // rho = |A^H A|_F / |A|_F, the root of the mean of sigma^2 weighted by sigma^2: equal to the
-  // spectral norm for flat and for rank-one spectra. Single precision is plenty for a scale.
-  const double inv = am > 0.0 ? 1.0 / am : 0.0;
-  float f2 = 0.f, g2 = 0.f;
-  for (int e = tid; e < N * N; e += kRootThreads) {
-    const int r = e / N, c = e - r * N;
-    float2 w = make_float2(0.f, 0.f);
-    if (r != c) {
-      const double2 z = tree_entry(P.in, r, c);
-      w = make_float2((float)(z.x * inv), (float)(z.y * inv));
-    }
-    a[e] = w;
-    f2 += w.x * w.x + w.y * w.y;
+  ea = __reduce_max_sync(0xffffffffu, ea);
+  ev = __reduce_max_sync(0xffffffffu, ev);
+  if (lane == 0) {
+    sh.ea[warp] = ea;
+    sh.ev[warp] = ev;
   }
   __syncthreads();
-  for (int e = tid; e < N * (N + 1) / 2; e += kRootThreads) {
+  for (int w = 0; w < kWarps; ++w) {
+    ea = max(ea, sh.ea[w]);
+    ev = max(ev, sh.ev[w]);
+  }
+  // entries and weights as floats below 2
+  float f2 = 0.f, am = 0.f, v2 = 0.f, vm = 0.f;
+  for (int e = tid; e < N * N; e += kThreads) {
+    const int r = e / N, c = e - r * N;
+    const double2 z = tree_entry(P.in, r, c);
+    const int ex = r == c ? (int)ev : (int)ea;
+    float2 w = make_float2(scaled_float(z.x, ex), scaled_float(z.y, ex));
+    const float m2 = w.x * w.x + w.y * w.y;
+    if (r == c) {
+      v2 += m2;
+      vm = fmaxf(vm, m2);
+      w = make_float2(0.f, 0.f);
+    } else {
+      f2 += m2;
+      am = fmaxf(am, m2);
+    }
+    sh.a[e] = w;
+  }
+  __syncthreads();
+  // rho = |A^H A|_F / |A|_F, the root of the mean of sigma^2 weighted by sigma^2: equal to the
+  // spectral norm for flat and for rank-one spectra
+  float g2 = 0.f;
+  for (int e = tid; e < N * (N + 1) / 2; e += kThreads) {
     int i, j;
-    tree_pair(e, i, j);  // i < j + 1: (i, j - 1) runs over the upper triangle
+    tree_pair(e, i, j);  // i < j: (i, j - 1) runs over the upper triangle
     --j;
     float re = 0.f, im = 0.f;
     for (int k = 0; k < N; ++k) {
-      const float2 x = a[k * N + i], y = a[k * N + j];  // conj(x) y
+      const float2 x = sh.a[k * N + i], y = sh.a[k * N + j];  // conj(x) y
       re += x.x * y.x + x.y * y.y;
       im += x.x * y.y - x.y * y.x;
     }
     g2 += (i == j ? 1.f : 2.f) * (re * re + im * im);
   }
-  const double F2 = block_reduce((double)f2, sh, dsum);
-  const double G2 = block_reduce((double)g2, sh, dsum);
+  f2 = warp_sum(f2);
+  g2 = warp_sum(g2);
+  v2 = warp_sum(v2);
+  am = warp_max(am);
+  vm = warp_max(vm);
+  if (lane == 0) {
+    sh.f[0][warp] = f2;
+    sh.f[1][warp] = g2;
+    sh.f[2][warp] = v2;
+    sh.f[3][warp] = am;
+    sh.f[4][warp] = vm;
+  }
+  __syncthreads();
   if (tid == 0) {
+    f2 = g2 = v2 = am = vm = 0.f;
+    for (int w = 0; w < kWarps; ++w) {
+      f2 += sh.f[0][w];
+      g2 += sh.f[1][w];
+      v2 += sh.f[2][w];
+      am = fmaxf(am, sh.f[3][w]);
+      vm = fmaxf(vm, sh.f[4][w]);
+    }
     // The loop weights enter g as exp of about |v|^2 / 2 spread over n pairs, hence |v|^2 / 8;
-    // no single entry may come near the format's limit.
-    double den = F2 > 0.0 ? am * sqrt(G2 / F2) : 0.0;
-    den = dmax(dmax(den, am), dmax(v2 * 0.125, vm * vm));
-    if (!(den > 0.0)) den = 1.0;
-    const double s = rsqrt(den);  // vertex scale, its mantissa cut to 5 bits: exact products
-    if (!(s > 1e-300 && s < 1e300)) bad = 1;
+    // |A_jk| and |v_j|^2 at most 0.8 keep A_jk + v_j v_k and 2 v_j v_k inside the format. den is
+    // in units of 2^top; a part that is far below the other does not count.
+    const int xa = (int)ea - 1023, xv = 2 * ((int)ev - 1023);
+    const float da = fmaxf(f2 > 0.f ? sqrtf(g2 / f2) : 0.f, 1.25f * sqrtf(am));
+    const float dv = fmaxf(v2 * 0.125f, 1.25f * vm);
+    int top = da > 0.f ? xa : xv;
+    if (dv > 0.f && xv > top) top = xv;
+    float den = fmaxf(da > 0.f && xa - top > -100 ? ldexpf(da, xa - top) : 0.f,
+                      dv > 0.f && xv - top > -100 ? ldexpf(dv, xv - top) : 0.f);
+    if (!(den > 0.f)) {
+      den = 1.f;
+      top = 0;
+    }
+    if (top & 1) {
+      den *= 2.f;
+      --top;
+    }
     int ex;
-    const double f = frexp(s, &ex);
-    s_m = (int)(f * 32.0);
-    s_e = ex - 1;  // scale = m / 16 * 2^e
-    if (s_m < 16 || s_m > 31) { s_m = 16; s_e = 0; bad = 1; }
-    // 1 / scale^N: (16 / m)^N in double-double by squaring, exponents apart
-    double bh = 16.0 / s_m, bl = __fma_rn(-bh, (double)s_m, 16.0) / s_m, h = 1.0, l = 0.0;
+    // vertex scale 1 / sqrt(den 2^top), a little below, its mantissa cut to 5 bits: exact products
+    const float f = frexpf(rsqrtf(den) * 0.999999f, &ex);
+    sh.m = (int)(f * 32.f);
+    sh.e = ex - 1 - top / 2;  // scale = m / 16 * 2^e
+    if (!(sh.m >= 16 && sh.m <= 31) || sh.e > 900 || sh.e < -900) {
+      sh.m = 16;
+      sh.e = 0;
+      bad = 1;
+    }
+  }
+  __syncthreads();
+  const int m = sh.m, e2 = sh.e;
+  if (tid == kThreads - 1) {  // 1 / scale^N: (16 / m)^N by squaring, exponents apart
+    double bh = 16.0 / m, bl = __fma_rn(-bh, (double)m, 16.0) / m, h = 1.0, l = 0.0;
     for (int k = N; k > 0; k >>= 1) {
       if (k & 1) dd_mul(h, l, bh, bl, h, l);
       dd_mul(bh, bl, bh, bl, bh, bl);
     }
-    TreeState& S = state[blockIdx.x];
-    for (int i = 0; i < 6; ++i) S.sum[i] = 0;
-    S.fac_hi = h;
-    S.fac_lo = l;
-    S.exp2 = -kTreeFrac - (P.n >= 3 ? P.n - 3 : 0) - s_e * N + (P.Ne - N);
-    S.done = 0;
-    S.bad = 0;
-    if (blockIdx.x == 0) *counter = 0;
+    S->fac_hi = h;
+    S->fac_lo = l;
+    S->exp2 = -kTreeFrac - (P.n >= 3 ? P.n - 3 : 0) - e2 * N + (P.Ne - N);
   }
-  __syncthreads();
-  const int m = s_m, e2 = s_e;
   // root level: vertex 2 p is index p, vertex 2 p + 1 is index p + n; padding vertices have no
   // edges, loop weight one and scale one half
-  Fxc* A = roots + P.root;
   const int polys = tree_polys(P.n), edges = P.Ne * (P.Ne - 1) / 2;
-  for (int p = tid; p < polys; p += kRootThreads) {
+  for (int p = tid; p < polys; p += kThreads) {
     int j, k;
     if (p < edges) tree_pair(p, j, k); else j = k = p - edges;
     const int r = (j & 1) ? (j >> 1) + P.n : (j >> 1), c = (k & 1) ? (k >> 1) + P.n : (k >> 1);
@@ -197,14 +250,28 @@ tree_root_kernel(const TreeProblem* __restrict__ table, TreeProblem one,
     } else if (j == k) {
       v.rh = 1 << (kTreeFrac - 1 - 2 * kLimbBits);
     }
-    fx_store(A + p, v);
+    fx_store(root.A + fx_at(p), v);
   }
   if (tid == 0) {
     Fxc v{};
     v.rh = 1 << (kTreeFrac - 2 * kLimbBits);
-    fx_store(A + polys, v);  // g = 1
+    fx_store(root.A + root.g, v);  // g = 1
+    for (int i = 0; i < 6; ++i) S->sum[i] = 0;
+    S->done = 0;
   }
-  if (__syncthreads_or((int)bad) && tid == 0) state[blockIdx.x].bad = 1;
+  const int any = __syncthreads_or((int)bad);
+  if (tid == 0) S->bad = any ? 1 : 0;
+}
+
+// kOne: one problem, passed as a kernel argument; otherwise a table in device memory.
+template <bool kOne>
+__global__ void __launch_bounds__(kRootThreads)
+tree_root_kernel(const TreeProblem* __restrict__ table, TreeProblem one, TreeState* __restrict__ state,
+                 unsigned* __restrict__ counter, char* __restrict__ levels) {
+  __shared__ RootShared sh;
+  const TreeProblem P = kOne ? one : table[blockIdx.x];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
+  tree_root<kRootThreads>(P, tree_level(levels + P.root, P.n, P.n, 1), state + blockIdx.x, sh);
 }
 
 // The problem's signed mean from its limb sums, to double.
@@ -214,7 +281,7 @@ __device__ void tree_result(const TreeProblem& P, TreeState* S, double* out, boo
   for (int c = 0; c < 2; ++c) {
     const long long h = (long long)__ldcg(&S->sum[3 * c]), m = (long long)__ldcg(&S->sum[3 * c + 1]),
                     l = (long long)__ldcg(&S->sum[3 * c + 2]);
-    __int128 r = (((__int128)h << kLimbBits) + m);
+    __int128 r = ((__int128)h << kLimbBits) + m;
     r = (r << kLimbBits) + l;
     const bool neg = r < 0;
     if (neg) r = -r;
@@ -238,34 +305,116 @@ __device__ void tree_result(const TreeProblem& P, TreeState* S, double* out, boo
   if (flags) out[2] = fail ? 1.0 : 0.0;
 }
 
+// One piece (tree_piece) per lane, four neighbouring lanes per coefficient; all lanes of a warp
+// call it together. A phase with few items is a chain of loads and products in each thread:
+// in pieces the chain is a quarter as long. `J`: tree_piece_job of `id`. Returns true in the lane
+// that holds a term in z.
+__device__ __forceinline__ TreeJob tree_piece_job(const TreePhase& s, int id, int& t) {
+  const int L = s.n - s.M + 1, q = id >> 2;
+  const bool active = q < L * s.items;
+  const int row = active ? tree_div(q, s.items, s.inv_items) : 0;
+  t = active ? L - 1 - row : 1 << 20;
+  return tree_job(s, 0, active ? q - row * s.items : 0);
+}
+__device__ __forceinline__ bool tree_piece_task(const TreeJob& J, int t, int sub, Fxc& z, unsigned& bad) {
+  const bool active = t <= J.top + 1;
+  FxAcc acc{0, 0, 0, 0, 0, 0};
+  Fxc old{};
+  if (active) {
+    old = tree_end_old(J, t, sub);
+    acc = tree_piece(J, t, sub);
+  }
+#pragma unroll
+  for (int d = 1; d <= 2; d <<= 1) {
+    acc.s2r += __shfl_xor_sync(0xffffffffu, acc.s2r, d);
+    acc.s1r += __shfl_xor_sync(0xffffffffu, acc.s1r, d);
+    acc.s0r += __shfl_xor_sync(0xffffffffu, acc.s0r, d);
+    acc.s2i += __shfl_xor_sync(0xffffffffu, acc.s2i, d);
+    acc.s1i += __shfl_xor_sync(0xffffffffu, acc.s1i, d);
+    acc.s0i += __shfl_xor_sync(0xffffffffu, acc.s0i, d);
+  }
+  if (!active) return false;
+  const Fxc v = fx_norm(acc, bad);
+  if (J.end != kDot) {
+    tree_end_part(J, t, sub, old, v, bad);
+    return false;
+  }
+  if (sub != 0) return false;
+  FxAcc dot = fx_acc_zero();
+  fx_mac(dot, v, old);
+  z = fx_norm(dot, bad);
+  return true;
+}
+
+// kOne: the phase of the one problem is set up on the host. Phases of at most `fine` pieces run in
+// pieces.
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
-tree_step_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int step,
-                 TreeState* __restrict__ state, Fxc* __restrict__ levels) {
-  const TreeProblem P = kOne ? one : table[blockIdx.y];
-  if (P.n - step <= P.m1) return;  // fewer steps than another problem's
-  const TreePhase s = tree_step_phase(levels + P.root, P.n, step);
-  const unsigned t = blockIdx.x * kTreeThreads + threadIdx.x;
+tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ TreePhase one, int step, int fine,
+                 TreeState* __restrict__ state, char* __restrict__ levels) {
+  __shared__ TreePhase many;
+  if (!kOne) {
+    if (table[blockIdx.y].n - step <= table[blockIdx.y].m1) return;  // fewer steps than another's
+    if (threadIdx.x == 0)
+      many = tree_whole_phase(levels + table[blockIdx.y].root, table[blockIdx.y].n, step);
+    __syncthreads();
+  }
+  const TreePhase& s = kOne ? one : many;
+  const int t = (int)(blockIdx.x * kTreeThreads + threadIdx.x);
   unsigned bad = 0;
-  if (t < tree_tasks(s)) {
-    int x;
-    Fxc z;
-    tree_task(s, t, x, z, bad);
+  int x;
+  Fxc z;
+  if (tree_pieces(s) <= fine) {
+    if ((t & ~31) < tree_pieces(s)) {
+      const TreeJob J = tree_piece_job(s, t, x);
+      tree_piece_task(J, x, t & 3, z, bad);
+    }
+  } else if (t < s.tasks) {
+    tree_task(s, 0, t, x, z, bad);
   }
   if (bad) atomicOr(&state[blockIdx.y].bad, 1u);
 }
 
+// Limb sums of the terms a thread met, one column per thread (64-bit atomics on one shared sum
+// were a third of a small problem's time).
+template <int kThreads>
+struct LimbSums {
+  long long v[6][kThreads];
+  __device__ void clear() {
+    for (int i = 0; i < 6; ++i) v[i][threadIdx.x] = 0;
+  }
+  __device__ void add(const Fxc& z, bool neg) {
+    const int sg = neg ? -1 : 1, t = threadIdx.x;
+    v[0][t] += sg * z.rh;
+    v[1][t] += sg * z.rm;
+    v[2][t] += sg * z.rl;
+    v[3][t] += sg * z.ih;
+    v[4][t] += sg * z.im;
+    v[5][t] += sg * z.il;
+  }
+  // After a barrier: warp w adds up the sums w, w + warps, ... into v[.][0].
+  __device__ void reduce() {
+    for (int i = threadIdx.x >> 5; i < 6; i += kThreads / 32) {
+      long long x = 0;
+      for (int t = threadIdx.x & 31; t < kThreads; t += 32) x += v[i][t];
+      for (int d = 16; d; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+      if ((threadIdx.x & 31) == 0) v[i][0] = x;
+    }
+  }
+};
+
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, unsigned total_units,
-            TreeState* __restrict__ state, unsigned* __restrict__ counter, Fxc* __restrict__ levels,
-            Fxc* __restrict__ scratch, size_t cta_elems, double* __restrict__ out, bool flags) {
+            TreeState* __restrict__ state, unsigned* __restrict__ counter, char* __restrict__ levels,
+            char* __restrict__ scratch, size_t cta_bytes, double* __restrict__ out, bool flags) {
   __shared__ TreeLevel lv[kMaxN / 2 + 2];  // levels m1 + 1 and m1: the unit and its parent
-  __shared__ unsigned long long sum[6];
+  __shared__ TreePhase phase[kMaxN / 2];
+  __shared__ LimbSums<kTreeThreads> sum;
   __shared__ unsigned s_unit;
   __shared__ int s_prob;
   const int tid = threadIdx.x;
-  Fxc* ws = scratch + (size_t)blockIdx.x * cta_elems;
+  char* ws = scratch + (size_t)blockIdx.x * cta_bytes;
   for (;;) {
     if (tid == 0) {
       const unsigned u = atomicAdd(counter, 1u);
@@ -277,7 +426,7 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
       }
       s_prob = lo;
     }
-    if (tid < 6) sum[tid] = 0;
+    sum.clear();
     __syncthreads();
     if (s_unit >= total_units) return;
     const int prob = s_prob;
@@ -285,31 +434,26 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
     const int n = P.n, m1 = P.m1, top = P.top, unit = (int)(s_unit - P.unit_base);
     if (tid == 0) tree_unit_levels(lv, levels + P.root, ws, n, m1, top, unit);
     __syncthreads();
+    // in shared memory because the accumulators leave no registers for them
+    if (tid < m1) phase[tid] = tree_unit_phase(lv, n, m1, top, unit, tid);
+    __syncthreads();
     unsigned bad = 0;
-    for (unsigned b = 0; b < 1u << (m1 - top); ++b) {
-      const int parity = __popc((unsigned)unit) + __popc(b);
+    for (unsigned b = 0; b < 1u << (m1 - top); ++b)
       for (int i = tree_first_phase(m1, top, b); i < m1; ++i) {
-        const TreePhase s = tree_unit_phase(lv, n, m1, top, unit, b, i);
-        const unsigned nt = tree_tasks(s);
-        for (unsigned t = tid; t < nt; t += kTreeThreads) {
+        const TreePhase& s = phase[i];
+        for (int t = tid; t < s.tasks; t += kTreeThreads) {
           int x;
           Fxc z;
-          if (tree_task(s, t, x, z, bad)) {
-            const int sg = ((__popc((unsigned)x) + parity) & 1) ? -1 : 1;
-            atomicAdd(&sum[0], (unsigned long long)(long long)(sg * z.rh));
-            atomicAdd(&sum[1], (unsigned long long)(long long)(sg * z.rm));
-            atomicAdd(&sum[2], (unsigned long long)(long long)(sg * z.rl));
-            atomicAdd(&sum[3], (unsigned long long)(long long)(sg * z.ih));
-            atomicAdd(&sum[4], (unsigned long long)(long long)(sg * z.im));
-            atomicAdd(&sum[5], (unsigned long long)(long long)(sg * z.il));
-          }
+          if (tree_task(s, b, t, x, z, bad))
+            sum.add(z, (__popc((unsigned)x) + __popc((unsigned)unit) + __popc(b)) & 1);
         }
         __syncthreads();
       }
-    }
     const int any = __syncthreads_or((int)bad);
     TreeState* S = state + prob;
-    if (tid < 6) atomicAdd(&S->sum[tid], sum[tid]);
+    sum.reduce();
+    __syncthreads();
+    if (tid < 6) atomicAdd(&S->sum[tid], (unsigned long long)sum.v[tid][0]);
     if (tid == 0 && any) atomicOr(&S->bad, 1u);
     __threadfence();
     __syncthreads();
@@ -323,7 +467,80 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
   }
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+// Small problems in one launch: a cluster of CTAs works a whole tree off breadth first, one
+// cluster barrier a level (a grid-wide step is a launch, 3 us; the levels of a small tree take
+// less). Its scratch holds every level.
+template <bool kOne>
+__global__ void __launch_bounds__(kRootThreads, 2)
+tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int first, int count,
+                  TreeState* __restrict__ state, char* __restrict__ scratch, size_t bytes,
+                  double* __restrict__ out, bool flags) {
+  __shared__ union {
+    RootShared root;
+    LimbSums<kRootThreads> sum;
+  } sh;
+  __shared__ TreePhase phase[kTreeSmallMax];
+  __shared__ unsigned s_bad;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), tid = threadIdx.x;
+  const int id = (int)blockIdx.x / C, clusters = (int)gridDim.x / C, stride = C * kRootThreads;
+  char* base = scratch + (size_t)id * bytes;
+  for (int p = first + id; p < first + count; p += clusters) {
+    const TreeProblem P = kOne ? one : table[p];
+    TreeState* S = state + p;
+    if (tid < P.n) phase[tid] = tree_whole_phase(base, P.n, tid);
+    if (tid == P.n) s_bad = 0;
+    if (rank == 0) tree_root<kRootThreads>(P, tree_level(base, P.n, P.n, 1), S, sh.root);
+    __syncthreads();
+    sh.sum.clear();
+    const int t0 = rank * kRootThreads + tid;
+    unsigned bad = 0;
+    int t;
+    TreeJob J = tree_piece_job(phase[0], t0, t);
+    cl.sync();
+    for (int i = 0; i < P.n; ++i) {
+      const TreePhase& s = phase[i];
+      const int pieces = tree_pieces(s);
+      int x;
+      Fxc z;
+      if (pieces <= 3 * stride) {
+        for (int q = t0; (q & ~31) < pieces; q += stride) {
+          if (q != t0) J = tree_piece_job(s, q, t);
+          if (tree_piece_task(J, t, q & 3, z, bad)) sh.sum.add(z, __popc((unsigned)J.node) & 1);
+        }
+      } else {
+        for (int q = t0; q < s.tasks; q += stride)
+          if (tree_task(s, 0, q, x, z, bad)) sh.sum.add(z, __popc((unsigned)x) & 1);
+      }
+      if (i == P.n - 1) {
+        if (bad) atomicOr(&s_bad, 1u);
+        __syncthreads();
+        sh.sum.reduce();
+      }
+      // the next phase's first job is worked out while the others arrive
+      auto token = cl.barrier_arrive();
+      if (i + 1 < P.n) J = tree_piece_job(phase[i + 1], t0, t);
+      cl.barrier_wait(std::move(token));
+    }
+    if (rank == 0) {
+      if (tid < 6) {
+        long long total = sh.sum.v[tid][0];
+        for (int r = 1; r < C; ++r) total += *cl.map_shared_rank(&sh.sum.v[tid][0], r);
+        S->sum[tid] = (unsigned long long)total;
+      }
+      if (tid == 6) {
+        unsigned b = s_bad;
+        for (int r = 1; r < C; ++r) b |= *cl.map_shared_rank(&s_bad, r);
+        if (b) S->bad = 1;
+      }
+      __syncthreads();
+      if (tid == 0) tree_result(P, S, out + 3 * (size_t)p, flags);
+    }
+    cl.sync();  // the other CTAs' sums were read
+  }
+}
+
+static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
@@ -337,40 +554,53 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
   std::stable_sort(T.order.begin(), T.order.end(), [&](int a, int b) { return Ns[a] > Ns[b]; });
   T.prob.resize(count);
   T.steps.clear();
+  auto pairs = [&](int q) { return std::max(4, Ns[T.order[q]] + (Ns[T.order[q]] & 1)) / 2; };
+  // in launch order: large, small
+  const int cluster_slots = 2 * dev.sm_count;
+  int alone = 0;
+  while (alone < count && pairs(count - 1 - alone) <= kTreeSmallMax) ++alone;
+  const int limit = alone * 8 <= cluster_slots ? kTreeSmallMax : kTreeSmallCrowd;
+  T.nbig = 0;
+  while (T.nbig < count && pairs(T.nbig) > limit) ++T.nbig;
+  const int nsmall = count - T.nbig;
+  T.cluster = T.clusters = 0;
+  T.small_bytes = 0;
+  if (nsmall > 0) {
+    // CTAs that the widest levels of the largest one can use, and that the GPU has
+    const int n = pairs(T.nbig);
+    T.cluster = n <= 3 ? 1 : (n <= 4 ? 4 : (n <= 6 ? 8 : 16));
+    while (T.cluster > 1 && nsmall * T.cluster > cluster_slots) T.cluster >>= 1;
+    T.clusters = std::min(nsmall, cluster_slots / T.cluster);
+    T.small_bytes = align256(tree_offset(1, n));
+  }
   const unsigned slots = (unsigned)(kTreeCtasPerSm * dev.sm_count);
   unsigned base = 0;
   size_t root = 0;
-  T.cta_elems = 1;
+  T.cta_bytes = 0;
+  T.fine = (int)slots * kTreeThreads / std::max(T.nbig, 1);  // pieces that still run all at once
   for (int q = 0; q < count; ++q) {
     TreeProblem& P = T.prob[q];
-    const int N = Ns[T.order[q]];
-    P.Ne = std::max(4, N + (N & 1));
-    P.n = P.Ne / 2;
-    const int n = P.n;
-    P.m1 = n;
-    P.top = std::min(n, kTreeTop);
-    if (n > 2) {
-      --P.m1;
-      const unsigned want = count == 1 ? 4 * slots : 2 * slots / (unsigned)count;
-      while (P.m1 > 2 && (unsigned)tree_width(P.m1, n) < want && n - P.m1 < (n > 24 ? 11 : 12)) --P.m1;
-    }
-    P.top = std::min(P.top, P.m1);
-    P.units = (unsigned)tree_width(P.m1, n);
+    const int n = pairs(q);
+    P.Ne = 2 * n;
+    P.n = n;
+    P.m1 = P.top = n;
+    P.units = 0;
     P.unit_base = base;
-    base += P.units;
     P.root = root;
-    root += tree_offset(P.m1 - 1, n);
-    T.cta_elems = std::max(T.cta_elems, tree_scratch(n, P.m1, P.top));
+    if (q >= T.nbig) continue;
+    P.m1 = n - 1;
+    const unsigned want = T.nbig == 1 ? 4 * slots : 2 * slots / (unsigned)T.nbig;
+    while (P.m1 > 2 && (unsigned)tree_width(P.m1, n) < want && n - P.m1 < (n > 24 ? 11 : 12)) --P.m1;
+    P.top = std::min(kTreeTop, P.m1);
+    P.units = (unsigned)tree_width(P.m1, n);
+    base += P.units;
+    root += align256(tree_offset(P.m1 - 1, n));
+    T.cta_bytes = std::max(T.cta_bytes, tree_scratch(n, P.m1, P.top));
     for (int i = 0; i < n - P.m1; ++i) {
       if ((int)T.steps.size() <= i) T.steps.push_back(TreePlan::Step{0, 0});
-      TreePhase s{};
-      s.kind = kTreeStep;
-      s.n = n;
-      s.M = n - i;
-      s.src.q = tree_width(n - i, n);
-      s.par.q = i > 0 ? tree_width(n - i + 1, n) : 0;
       T.steps[i].problems = q + 1;
-      T.steps[i].tasks = std::max(T.steps[i].tasks, tree_tasks(s));
+      const TreePhase s = tree_whole_phase(nullptr, n, i);
+      T.steps[i].tasks = std::max(T.steps[i].tasks, tree_pieces(s) <= T.fine ? tree_pieces(s) : s.tasks);
     }
   }
   T.total_units = base;
@@ -380,8 +610,9 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
   T.off_state = off; off = align256(off + sizeof(TreeState) * (size_t)count);
   T.off_counter = off; off = align256(off + sizeof(unsigned));
   T.off_out = off; off = align256(off + 3 * sizeof(double) * (size_t)count);
-  T.off_root = off; off = align256(off + sizeof(Fxc) * root);
-  T.off_cta = off; off = align256(off + sizeof(Fxc) * T.cta_elems * (size_t)T.blocks);
+  T.off_root = off; off = align256(off + root);
+  T.off_cta = off;  // the two kinds of scratch are not used at the same time
+  off = align256(off + std::max(T.cta_bytes * (size_t)T.blocks, T.small_bytes * (size_t)T.clusters));
   T.bytes = off;
   return cudaSuccess;
 }
@@ -397,34 +628,79 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
   const int count = (int)plan.prob.size();
   if (count == 0) return cudaSuccess;
   char* b = static_cast<char*>(ws);
-  const TreeProblem* table = count > 1 ? reinterpret_cast<const TreeProblem*>(b + plan.off_prob) : nullptr;
+  const bool one = count == 1, flags = value == nullptr;
+  const TreeProblem* table = one ? nullptr : reinterpret_cast<const TreeProblem*>(b + plan.off_prob);
   TreeState* state = reinterpret_cast<TreeState*>(b + plan.off_state);
   unsigned* counter = reinterpret_cast<unsigned*>(b + plan.off_counter);
-  Fxc* roots = reinterpret_cast<Fxc*>(b + plan.off_root);
-  Fxc* scratch = reinterpret_cast<Fxc*>(b + plan.off_cta);
+  char* levels = b + plan.off_root;
+  char* scratch = b + plan.off_cta;
   double* out = value ? value : reinterpret_cast<double*>(b + plan.off_out);
-  const bool one = count == 1;
   const TreeProblem& p0 = plan.prob[0];
-  if (one)
-    tree_root_kernel<true><<<1, kRootThreads, 0, st>>>(table, p0, state, counter, roots);
-  else
-    tree_root_kernel<false><<<count, kRootThreads, 0, st>>>(table, p0, state, counter, roots);
-  for (size_t i = 0; i < plan.steps.size(); ++i) {
-    const dim3 grid((plan.steps[i].tasks + kTreeThreads - 1) / kTreeThreads, plan.steps[i].problems);
+  cudaError_t e = cudaSuccess;
+  if (plan.nbig > 0) {
     if (one)
-      tree_step_kernel<true><<<grid, kTreeThreads, 0, st>>>(table, p0, (int)i, state, roots);
+      tree_root_kernel<true><<<1, kRootThreads, 0, st>>>(table, p0, state, counter, levels);
     else
-      tree_step_kernel<false><<<grid, kTreeThreads, 0, st>>>(table, p0, (int)i, state, roots);
+      tree_root_kernel<false><<<plan.nbig, kRootThreads, 0, st>>>(table, p0, state, counter, levels);
+    for (int i = 0; i < (int)plan.steps.size(); ++i) {
+      const dim3 grid((plan.steps[i].tasks + kTreeThreads - 1) / kTreeThreads, plan.steps[i].problems);
+      const TreePhase s = tree_whole_phase(levels + p0.root, p0.n, i);
+      if (one)
+        tree_step_kernel<true><<<grid, kTreeThreads, 0, st>>>(table, s, i, plan.fine, state, levels);
+      else
+        tree_step_kernel<false><<<grid, kTreeThreads, 0, st>>>(table, s, i, plan.fine, state, levels);
+    }
+    if (one)
+      tree_kernel<true><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, 1, plan.total_units, state, counter,
+                                                              levels, scratch, plan.cta_bytes, out, flags);
+    else
+      tree_kernel<false><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, plan.nbig, plan.total_units, state,
+                                                               counter, levels, scratch, plan.cta_bytes, out,
+                                                               flags);
+    e = cudaGetLastError();
   }
-  if (one)
-    tree_kernel<true><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, count, plan.total_units, state,
-                                                            counter, roots, scratch, plan.cta_elems,
-                                                            out, value == nullptr);
-  else
-    tree_kernel<false><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, count, plan.total_units, state,
-                                                             counter, roots, scratch, plan.cta_elems,
-                                                             out, value == nullptr);
-  return cudaGetLastError();
+  if (e == cudaSuccess && plan.nbig < count) {
+    const auto k = one ? tree_small_kernel<true> : tree_small_kernel<false>;
+    if (plan.cluster > 8) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(plan.clusters * plan.cluster));
+    cfg.blockDim = dim3(kRootThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)plan.cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, k, table, p0, plan.nbig, count - plan.nbig, state, scratch, plan.small_bytes,
+                           out, flags);
+  }
+  return e;
+}
+
+cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st, double* out3,
+                     std::vector<int>* again) {
+  const size_t count = plan->prob.size();
+  std::vector<double> res(3 * count);
+  cudaError_t e = tree_stage(plan, in, ws, st);
+  if (e == cudaSuccess) e = tree_launch(*plan, ws, st);
+  if (e == cudaSuccess && count > 0)
+    e = cudaMemcpyAsync(res.data(), static_cast<char*>(ws) + plan->off_out, sizeof(double) * res.size(),
+                        cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
+  for (size_t q = 0; q < count; ++q) {
+    const int p = plan->order[q];
+    if (res[3 * q + 2] != 0.0) again->push_back(p);
+    out3[3 * (size_t)p] = res[3 * q];
+    out3[3 * (size_t)p + 1] = res[3 * q + 1];
+    out3[3 * (size_t)p + 2] = 0.0;
+  }
+  std::sort(again->begin(), again->end());
+  return cudaSuccess;
 }
 
 const unsigned* tree_flag(const TreePlan& plan, void* ws) {

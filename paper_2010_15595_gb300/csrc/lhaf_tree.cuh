@@ -24,21 +24,22 @@
 // subset sum cancels by 10^7..10^12.
 //
 // Arithmetic. Products of polynomials are sums of products with no division, so they run in
-// fixed point: a real number is an 84-bit integer times 2^-81, held as three 28-bit limbs
-// with signs (h 2^56 + m 2^28 + l). GB300 issues 64 32x32+64-bit integer multiply-adds per SM
-// and clock (measured 18.7e12/s), a limb product is at most 2^54, and up to 2^9 of them add
-// up in 64 bits without a carry, so a whole convolution accumulates exactly and is normalised
-// once. Six limb products per real product (the three below 2^-81 are dropped) make 24
-// multiply-adds per complex one: 0.78e12 complex multiply-adds/s, against 0.17e12/s for
-// triple-float (216 FP32 instructions) and 0.15e12/s for FP64. Fixed point needs a scale: the
-// matrix is scaled by one factor such that its root-mean-fourth singular value is about one,
-// which keeps the coefficients of every matrix tried between 2^-10 and 1.5 (the format holds
-// |x| < 4). Overflow anywhere, or a result so small that the 2^-81 resolution could show, sets
-// a flag and the caller evaluates the problem by the subset sum instead.
+// fixed point: a real number is an integer times 2^-81, held as three limbs with signs,
+// h 2^54 + m 2^27 + l, |m|, |l| <= 2^26, |h| < 2^29. The limb products of a whole convolution
+// add up in 64 bits, so it accumulates exactly and is normalised once. Six limb products per real
+// product (the three below 2^-81 are dropped) make 24 32x32+64-bit integer multiply-adds per
+// complex one: 0.35e12 complex multiply-adds/s with operands from L1, against 0.17e12/s at best
+// for triple-float (216 FP32 instructions) and 0.15e12/s for FP64. (The integer multiply-add
+// issues every 2 cycles when it repeats its operands, 18.7e12/s, and every 4.4 in this code; its
+// operand fetch is the limit of the whole evaluation.) Fixed point needs a scale: the matrix is
+// scaled by one factor such that its root-mean-fourth singular value is about one, which keeps
+// the coefficients of every matrix tried between 2^-10 and 2.5 (the format holds |x| < 4).
+// Overflow anywhere, or a result so small that the 2^-81 resolution could show, sets a flag and
+// the caller evaluates the problem by the subset sum instead.
 //
 // The code of one level is a function of (level, task number) that reads the level's nodes
 // and writes the next level's, so it compiles for the host as well and is checked there
-// against the definition, with every index bounds-checked.
+// against the definition.
 #pragma once
 
 #include <cstddef>
@@ -53,113 +54,118 @@
 
 namespace gbsh {
 
-constexpr int kTreeFrac = 81;        // value = integer * 2^-81
-constexpr int kLimbBits = 28;
+constexpr int kTreeFrac = 81;  // value = integer * 2^-81
+constexpr int kLimbBits = 27;
+constexpr int kLimbHalf = 1 << (kLimbBits - 1);
+constexpr int kLimbMask = (1 << kLimbBits) - 1;
 
-// A complex fixed-point number: limbs of the real and the imaginary part (32 bytes, so that
-// an element is two 16-byte loads).
-struct alignas(16) Fxc {
-  int rh, rm, rl, ih;
-  int im, il, pad0, pad1;
+// A complex fixed-point number: limbs of the real and the imaginary part.
+struct Fxc {
+  int rh, rm, rl, ih, im, il;
 };
 
-// 64-bit limb-product sums of one complex accumulator, by weight: s2 2^112, s1 2^84, s0 2^56
-// (in units of 2^-162).
+// In memory a row of numbers lies in blocks of 32: 32 (rh, rm), 32 (rl, ih), 32 (im, il) pairs.
+// A warp that reads 32 neighbours then takes three 256-byte runs, where 24- or 32-byte
+// structures cost it five times the L1 wavefronts. Numbers are addressed by bytes.
+GBSH_HD constexpr int fx_at(int i) { return (i >> 5) * 768 + (i & 31) * 8; }
+GBSH_HD constexpr int fx_row(int count) { return ((count + 31) >> 5) * 768; }
+
+GBSH_HD Fxc fx_load(const char* p) {
+#ifdef __CUDA_ARCH__
+  const int2 a = *reinterpret_cast<const int2*>(p), b = *reinterpret_cast<const int2*>(p + 256),
+             c = *reinterpret_cast<const int2*>(p + 512);
+  return Fxc{a.x, a.y, b.x, b.y, c.x, c.y};
+#else
+  const int *a = reinterpret_cast<const int*>(p), *b = a + 64, *c = a + 128;
+  return Fxc{a[0], a[1], b[0], b[1], c[0], c[1]};
+#endif
+}
+GBSH_HD void fx_store(char* p, const Fxc& v) {
+#ifdef __CUDA_ARCH__
+  *reinterpret_cast<int2*>(p) = make_int2(v.rh, v.rm);
+  *reinterpret_cast<int2*>(p + 256) = make_int2(v.rl, v.ih);
+  *reinterpret_cast<int2*>(p + 512) = make_int2(v.im, v.il);
+#else
+  int *a = reinterpret_cast<int*>(p), *b = a + 64, *c = a + 128;
+  a[0] = v.rh, a[1] = v.rm, b[0] = v.rl, b[1] = v.ih, c[0] = v.im, c[1] = v.il;
+#endif
+}
+
+// 64-bit limb-product sums of one complex accumulator, by weight: s2 2^108, s1 2^81, s0 2^54
+// (in units of 2^-162). They start at half a unit of the next limb, which turns the cuts in
+// fx_norm into roundings to the nearest.
 struct FxAcc {
   long long s2r, s1r, s0r, s2i, s1i, s0i;
 };
-
-GBSH_HD FxAcc fx_acc_zero() { return FxAcc{0, 0, 0, 0, 0, 0}; }
-
-GBSH_HD Fxc fx_load(const Fxc* p) {
-#ifdef __CUDA_ARCH__
-  const int4 a = reinterpret_cast<const int4*>(p)[0];
-  const int2 b = reinterpret_cast<const int2*>(p)[2];
-  return Fxc{a.x, a.y, a.z, a.w, b.x, b.y, 0, 0};
-#else
-  return *p;
-#endif
+GBSH_HD FxAcc fx_acc_zero() {
+  return FxAcc{kLimbHalf, kLimbHalf, kLimbHalf, kLimbHalf, kLimbHalf, kLimbHalf};
 }
-GBSH_HD void fx_store(Fxc* p, const Fxc& v) {
-#ifdef __CUDA_ARCH__
-  reinterpret_cast<int4*>(p)[0] = make_int4(v.rh, v.rm, v.rl, v.ih);
-  reinterpret_cast<int2*>(p)[2] = make_int2(v.im, v.il);
-#else
-  *p = v;
-#endif
+// (s2, s1, s0) += a b of two real numbers. The limb products of weight 2^27 and 1 are below the
+// result's resolution.
+GBSH_HD void fx_mac1(long long& s2, long long& s1, long long& s0, int ah, int am, int al, int bh, int bm, int bl) {
+  s2 += (long long)ah * bh;
+  s1 += (long long)ah * bm;
+  s0 += (long long)ah * bl;
+  s1 += (long long)am * bh;
+  s0 += (long long)am * bm;
+  s0 += (long long)al * bh;
 }
-
-// acc += a * b. The limb products of weight 2^28 and 1 are below the result's resolution.
+// acc += a * b. Three real products a complex one (Gauss) would be 18 multiply-adds instead of
+// 24, but the third set of sums costs registers: no faster with 128 registers a thread and
+// slower with fewer.
 GBSH_HD void fx_mac(FxAcc& s, const Fxc& a, const Fxc& b) {
-  const int nh = -a.ih, nm = -a.im, nl = -a.il;
-  s.s2r += (long long)a.rh * b.rh;
-  s.s2r += (long long)nh * b.ih;
-  s.s1r += (long long)a.rh * b.rm;
-  s.s1r += (long long)a.rm * b.rh;
-  s.s1r += (long long)nh * b.im;
-  s.s1r += (long long)nm * b.ih;
-  s.s0r += (long long)a.rh * b.rl;
-  s.s0r += (long long)a.rl * b.rh;
-  s.s0r += (long long)a.rm * b.rm;
-  s.s0r += (long long)nh * b.il;
-  s.s0r += (long long)nl * b.ih;
-  s.s0r += (long long)nm * b.im;
-  s.s2i += (long long)a.rh * b.ih;
-  s.s2i += (long long)a.ih * b.rh;
-  s.s1i += (long long)a.rh * b.im;
-  s.s1i += (long long)a.rm * b.ih;
-  s.s1i += (long long)a.ih * b.rm;
-  s.s1i += (long long)a.im * b.rh;
-  s.s0i += (long long)a.rh * b.il;
-  s.s0i += (long long)a.rl * b.ih;
-  s.s0i += (long long)a.rm * b.im;
-  s.s0i += (long long)a.ih * b.rl;
-  s.s0i += (long long)a.il * b.rh;
-  s.s0i += (long long)a.im * b.rm;
+  fx_mac1(s.s2r, s.s1r, s.s0r, a.rh, a.rm, a.rl, b.rh, b.rm, b.rl);
+  fx_mac1(s.s2i, s.s1i, s.s0i, a.rh, a.rm, a.rl, b.ih, b.im, b.il);
+  fx_mac1(s.s2r, s.s1r, s.s0r, -a.ih, -a.im, -a.il, b.ih, b.im, b.il);
+  fx_mac1(s.s2i, s.s1i, s.s0i, a.ih, a.im, a.il, b.rh, b.rm, b.rl);
 }
 
-GBSH_HD int sext28(long long x) { return (int)((unsigned)x << 4) >> 4; }
-
-// The accumulated real number rounded to the format; bad |= it does not fit (|x| < 2).
-GBSH_HD void fx_norm(long long s2, long long s1, long long s0, int& h, int& m, int& l, unsigned& bad) {
-  bad |= (unsigned)((unsigned long long)(s2 + (1ll << 51)) >> 52);
-  // in units of 2^-81: s2 2^31 + s1 2^3 + s0 2^-25
-  const long long lo = ((s1 & ((1ll << 25) - 1)) << 3) + ((s0 + (1ll << 24)) >> 25);
-  l = sext28(lo);
-  const long long v = (long long)((unsigned long long)s2 << 3) + (s1 >> 25) + ((lo - l) >> 28);
-  m = sext28(v);
-  h = (int)((v - m) >> 28);
+// The accumulated real number rounded to the format: s2 2^27 + s1 + s0 2^-27; bad |= |x| >= 4.
+// (s2 itself holds |x| < 512: 32 products of numbers at the limit.)
+GBSH_HD void fx_norm1(long long s2, long long s1, long long s0, int& h, int& m, int& l, unsigned& bad) {
+  const long long t = s1 + (s0 >> kLimbBits);
+  l = ((int)t & kLimbMask) - kLimbHalf;
+  const long long v = s2 + (t >> kLimbBits);
+  m = ((int)v & kLimbMask) - kLimbHalf;
+  h = (int)(v >> kLimbBits);
+  bad |= (unsigned)((int)(v >> 32) + (1 << 24)) >> 25;
 }
 GBSH_HD Fxc fx_norm(const FxAcc& s, unsigned& bad) {
-  Fxc r{};
-  fx_norm(s.s2r, s.s1r, s.s0r, r.rh, r.rm, r.rl, bad);
-  fx_norm(s.s2i, s.s1i, s.s0i, r.ih, r.im, r.il, bad);
+  Fxc r;
+  fx_norm1(s.s2r, s.s1r, s.s0r, r.rh, r.rm, r.rl, bad);
+  fx_norm1(s.s2i, s.s1i, s.s0i, r.ih, r.im, r.il, bad);
   return r;
 }
 
-// (h, m, l) = a + sg b, carries propagated; bad |= |result| >= 4.
-GBSH_HD void fx_add1(int ah, int am, int al, int bh, int bm, int bl, int sg, int& h, int& m, int& l,
-                     unsigned& bad) {
-  const int x = al + sg * bl;
-  l = sext28(x);
-  const int y = am + sg * bm + ((x - l) >> 28);
-  m = sext28(y);
-  h = ah + sg * bh + ((y - m) >> 28);
-  bad |= (unsigned)(h + (1 << 27)) >> 28;
+// (h, m, l) from limbs with carries to propagate; bad |= |x| >= 4.
+GBSH_HD void fx_carry(int xh, int xm, int xl, int& h, int& m, int& l, unsigned& bad) {
+  const int a = xl + kLimbHalf;
+  l = (a & kLimbMask) - kLimbHalf;
+  const int b = xm + kLimbHalf + (a >> kLimbBits);
+  m = (b & kLimbMask) - kLimbHalf;
+  h = xh + (b >> kLimbBits);
+  bad |= (unsigned)(h + (1 << 29)) >> 30;
 }
-GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, int sg, unsigned& bad) {
-  Fxc r{};
-  fx_add1(a.rh, a.rm, a.rl, b.rh, b.rm, b.rl, sg, r.rh, r.rm, r.rl, bad);
-  fx_add1(a.ih, a.im, a.il, b.ih, b.im, b.il, sg, r.ih, r.im, r.il, bad);
+GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, unsigned& bad) {
+  Fxc r;
+  fx_carry(a.rh + b.rh, a.rm + b.rm, a.rl + b.rl, r.rh, r.rm, r.rl, bad);
+  fx_carry(a.ih + b.ih, a.im + b.im, a.il + b.il, r.ih, r.im, r.il, bad);
+  return r;
+}
+GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, unsigned& bad) {
+  Fxc r;
+  fx_carry(a.rh - b.rh, a.rm - b.rm, a.rl - b.rl, r.rh, r.rm, r.rl, bad);
+  fx_carry(a.ih - b.ih, a.im - b.im, a.il - b.il, r.ih, r.im, r.il, bad);
   return r;
 }
 
-// acc0, acc1 += coefficients t0, t0 + 1 of the polynomial product a * b, a[u] at a + u sa, b[u]
-// at b + u sb; t0 = -1 leaves acc0 alone. t0 + 1 must not exceed the last coefficient of either
+// acc0, acc1 += coefficients t0, t0 + 1 of the polynomial product a * b, coefficient u at a + u sa
+// and b + u sb; t0 = -1 leaves acc0 alone. t0 + 1 must not exceed the last coefficient of either
 // factor. Two coefficients a task: each step loads one new element of each factor for two
 // multiply-adds (b in a sliding window of two). Four would halve the loads, but with the
-// accumulators of four (48 registers) the code spilled and outgrew the instruction cache.
-GBSH_HD void fx_conv2(FxAcc& acc0, FxAcc& acc1, const Fxc* a, int sa, const Fxc* b, int sb, int t0) {
+// accumulators of four (48 registers) the code spilled and outgrew the instruction cache
+// (N = 40: 9.0 ms against 5.7 ms).
+GBSH_HD void fx_conv2(FxAcc& acc0, FxAcc& acc1, const char* a, int sa, const char* b, int sb, int t0) {
   b += (ptrdiff_t)(t0 + 1) * sb;
   Fxc w1 = fx_load(b), w0{};
   int u = t0 + 1;  // steps before the last one
@@ -204,41 +210,47 @@ GBSH_HD void fx_conv2(FxAcc& acc0, FxAcc& acc1, const Fxc* a, int sa, const Fxc*
 // Level M holds nodes with M pairs left: r = 2M vertices, L = n - M + 1 coefficients per
 // polynomial. A node's polynomials are the A_jk, j < k < r, at k (k - 1) / 2 + j (so that
 // eliminating the last pair leaves the others in place) and the loop weights v_j at
-// r (r - 1) / 2 + j. Coefficient u of polynomial p of node x is A[(u ld + x) P + p]; g and
-// h = A_ab + v_a v_b (of the pair that is eliminated next) are at [u ld + x].
+// r (r - 1) / 2 + j: P(M) in all. Coefficient u of the polynomials of all nodes is a row, number
+// x P + p of it belongs to node x; the rows of g and of h = A_ab + v_a v_b (of the pair that is
+// eliminated next) have one number per node.
 GBSH_HD constexpr int tree_polys(int M) { return M * (2 * M + 1); }
 
 struct TreeLevel {
-  Fxc* A;
-  Fxc* g;
-  Fxc* h;
-  int q;   // nodes, from the pointers on
-  int ld;  // nodes stored side by side
+  char* A;           // row 0 of the A_jk and v_j
+  int g, h;          // bytes from there to the rows of g and h
+  int sA, sg, sh;    // bytes from row to row
+  int q, x0;         // nodes x0 .. x0 + q - 1
 };
 
-// Elements of a level of q nodes (level 2 holds the eight w and v v polynomials in place of h).
-GBSH_HD size_t tree_level_elems(int M, int n, int q) {
-  return (size_t)q * (n - M + 1) * (tree_polys(M) + 1 + (M == 2 ? 8 : 1));
+// Level 2 holds the eight w and v v polynomials per node in place of h.
+GBSH_HD size_t tree_level_bytes(int M, int n, int q) {
+  return (size_t)(n - M + 1) * (fx_row(q * tree_polys(M)) + fx_row(q) + fx_row(M == 2 ? 8 * q : q));
 }
-GBSH_HD TreeLevel tree_level(Fxc* base, int M, int n, int q) {
-  const size_t L = n - M + 1;
+GBSH_HD TreeLevel tree_level(char* base, int M, int n, int q) {
+  const int L = n - M + 1;
   TreeLevel v;
+  v.sA = fx_row(q * tree_polys(M));
+  v.sg = fx_row(q);
+  v.sh = fx_row(M == 2 ? 8 * q : q);
   v.A = base;
-  v.g = base + (size_t)q * L * tree_polys(M);
-  v.h = v.g + (size_t)q * L;
-  v.q = v.ld = q;
+  v.g = L * v.sA;
+  v.h = v.g + L * v.sg;
+  v.q = q;
+  v.x0 = 0;
   return v;
 }
 // Node x of a level as a level of one node.
-GBSH_HD TreeLevel tree_node(const TreeLevel& v, int M, int x) {
-  return TreeLevel{v.A + (size_t)x * tree_polys(M), v.g + x, v.h + (M == 2 ? 8 * x : x), 1, v.ld};
+GBSH_HD TreeLevel tree_node(TreeLevel v, int x) {
+  v.x0 += x;
+  v.q = 1;
+  return v;
 }
-// Nodes of level M of the whole tree, and the element offset of that level when the levels
+// Nodes of level M of the whole tree, and the byte offset of that level when the levels
 // n, n - 1, ... follow each other.
 GBSH_HD int tree_width(int M, int n) { return n - M < 2 ? 1 : 1 << (n - M - 1); }
 GBSH_HD size_t tree_offset(int M, int n) {
   size_t off = 0;
-  for (int m = n; m > M; --m) off += tree_level_elems(m, n, tree_width(m, n));
+  for (int m = n; m > M; --m) off += tree_level_bytes(m, n, tree_width(m, n));
   return off;
 }
 
@@ -254,14 +266,21 @@ GBSH_HD void tree_pair(int p, int& j, int& k) {
   j = p - k * (k - 1) / 2;
 }
 
+// a / b for 0 <= a < 2^23, b > 0, inv = 1 / b in single precision.
+GBSH_HD int tree_div(int a, int b, float inv) {
+  int x = (int)((float)a * inv);
+  if (x * b > a) --x;
+  if ((x + 1) * b <= a) ++x;
+  return x;
+}
+
 // One phase of a node set's way down the tree; its tasks are independent of each other.
 //   step    one elimination, level M (src) to level M - 1 (dst): both children of every node
 //           x, 2 x with + and 2 x + 1 with -, or (`single`, at the root) the + child alone. The
 //           g of src's nodes are made here too, from their parents' (par, one level up), and h
 //           of src's nodes: both lag a level so that a level has no chain of products. `psign` =
-//           0: src holds both children of each node of par, and `gsel` tells by how many nodes
-//           its pointers are past the first; +-1: src is that child of par's one node. At the
-//           root (M = n) g is one and has no parent.
+//           0: src's storage holds both children of each node of par; +-1: src is that child of
+//           par's one node. At the root (M = n) g is one and has no parent.
 //   last1   level 2 (src): w_jk = A_jk + v_j v_k at 8 x + p (p the pair's number), -2 v0 v1 at
 //           8 x + 6 and v2 v3 at 8 x + 7, in place of h; and g of the level's nodes.
 //   last2   level 2 (src): the products w01 w23, w02 w13, w03 w12, -2 v0 v1 v2 v3 of a node,
@@ -269,207 +288,310 @@ GBSH_HD void tree_pair(int p, int& j, int& k) {
 enum TreeKind { kTreeStep, kTreeLast1, kTreeLast2 };
 struct TreePhase {
   TreeLevel src, dst, par;
-  int kind, n, M, psign, gsel;
+  int kind, n, M, psign;
   bool single;
+  int src_bit, par_bit;  // a level walked depth first: its node is this bit of the walk's number;
+                         // -1: its nodes are those of src and par
+  // set by tree_ready
+  int nmain, items, tasks;
+  float inv_items, inv_node;
 };
 
-GBSH_HD int tree_items(const TreePhase& s) {
-  if (s.kind == kTreeLast2) return 4 * s.src.q;
-  const int g = s.M < s.n ? s.par.q : 0;
-  return s.kind == kTreeStep ? s.src.q * (tree_polys(s.M - 1) + 1) + g : 6 * s.src.q + g;
-}
-GBSH_HD unsigned tree_tasks(const TreePhase& s) {
-  return (unsigned)((s.n - s.M + 2) / 2 * tree_items(s));
+// A task makes coefficients in twos: a tile near the top and its mirror tile near the bottom of
+// an item's triangle of products, so that all tasks of a phase cost the same.
+GBSH_HD void tree_ready(TreePhase& s) {
+  const int L = s.n - s.M + 1, g = s.M < s.n ? s.par.q : 0;
+  const int per = s.kind == kTreeStep ? tree_polys(s.M - 1) : (s.kind == kTreeLast1 ? 6 : 4);
+  s.nmain = s.src.q * (s.kind == kTreeStep ? per + 1 : per);
+  s.items = s.nmain + (s.kind == kTreeLast2 ? 0 : g);
+  s.tasks = ((L + 1) / 2 + 1) / 2 * s.items;
+  s.inv_items = 1.0f / (float)s.items;
+  s.inv_node = 1.0f / (float)per;
 }
 
-// Runs one task. In phase last2 returns true with a part of node `node`'s term in z.
-GBSH_HD bool tree_task(const TreePhase& s, unsigned task, int& node, Fxc& z, unsigned& bad) {
-  const int M = s.M, L = s.n - M + 1, q = s.src.q, ld = s.src.ld, r = 2 * M;
-  const int items = tree_items(s);
-  const int tile = (int)(task / (unsigned)items), it = (int)(task - (unsigned)tile * (unsigned)items);
-  int t0 = L - 2 - 2 * tile;  // the costliest coefficients first
-  // The task: coefficients t0, t0 + 1 of f0 * f1 (+ f2 * f3), then one of three ends.
-  const Fxc *f0, *f1, *f2 = nullptr, *f3 = nullptr;
-  int stride;
-  enum { kChild, kStore, kDot } end;
-  const Fxc* old;      // kChild: the polynomial to which +- x (product) is added; kStore: (product)
-  int ostride = 0;
-  Fxc* dst = nullptr;
-  int dstride = 0, twin = 0;  // kChild: the - child's distance (0: one child, sign `sg`)
-  int sg = 1, Lold = L, extra = 0;
-  const int nmain = s.kind == kTreeStep ? q * (tree_polys(M - 1) + 1) : 6 * q;
+// An item of a phase: the products f0 * f1 (+ g0 * g1) and what becomes of them. Byte offsets
+// from fb and db instead of pointers: the accumulators leave few registers.
+enum TreeEnd { kChild, kStore, kDot };
+struct TreeJob {
+  const char* fb;
+  char* db;
+  int f0, f1, g0, g1;  // factors; g0 < 0: one product
+  int sa, sb;          // row strides of the factors
+  TreeEnd end;
+  int old, so;         // kChild: the polynomial to which +- x (product) is added; kStore: (product)
+  int dst, twin, sd;   // kChild: the + and the - child (or one, the - child if `neg`)
+  int top, last;       // two below the number of coefficients; last coefficient of `old`
+  int node;
+  bool neg;
+};
+GBSH_HD TreeJob tree_job(const TreePhase& s, unsigned walk, int it) {
+  const int xs = s.src_bit < 0 ? s.src.x0 : (int)(walk >> s.src_bit) & 1;
+  const int L = s.n - s.M + 1;
+  TreeJob J;
+  J.fb = s.src.A;
+  J.db = s.src.A;
+  J.g0 = J.g1 = -1;
+  J.dst = 0;
+  J.twin = -1;
+  J.sd = 0;
+  J.top = L - 2;
+  J.last = L - 1;
+  J.neg = false;
+  J.node = 0;
   if (s.kind == kTreeLast2) {
     // pairs (01,23) = (0,5), (02,13) = (1,4), (03,12) = (3,2), then (6,7)
-    const int x = it >> 2, c = it & 3;
-    stride = ld * 8;
-    const Fxc* w = s.src.h + (ptrdiff_t)x * 8;
-    f0 = w + (c == 0 ? 0 : (c == 1 ? 1 : (c == 2 ? 3 : 6)));
-    f1 = w + (c == 3 ? 7 : (c == 2 ? 2 : 5 - c));
-    end = kDot;
-    old = s.src.g + x;
-    ostride = ld;
-    node = x;
-  } else if (it >= nmain) {  // g' = g +- x g h of node(s) of src
-    const int x = it - nmain;
-    --t0;
-    if (t0 < -1) return false;
-    stride = s.par.ld;
-    f0 = s.par.g + x;
-    f1 = s.par.h + x;
-    end = kChild;
-    old = f0;
-    ostride = stride;
-    Lold = L - 1;
-    sg = s.psign;
-    twin = s.psign == 0 ? 1 : 0;
-    dst = s.psign == 0 ? s.src.g - s.gsel + 2 * x : s.src.g;
-    dstride = ld;
+    const int x = it >> 2, c = it & 3, at = 8 * (xs + x);
+    J.sa = J.sb = s.src.sh;
+    J.f0 = s.src.h + fx_at(at + (c == 0 ? 0 : (c == 1 ? 1 : (c == 2 ? 3 : 6))));
+    J.f1 = s.src.h + fx_at(at + (c == 3 ? 7 : (c == 2 ? 2 : 5 - c)));
+    J.end = kDot;
+    J.old = s.src.g + fx_at(xs + x);
+    J.so = s.src.sg;
+    J.node = x;
+  } else if (it >= s.nmain) {  // g' = g +- x g h of node(s) of src
+    const int x = it - s.nmain;
+    const int xp = (s.par_bit < 0 ? s.par.x0 : (int)(walk >> s.par_bit) & 1) + x;
+    J.fb = s.par.A;
+    --J.top;
+    --J.last;
+    J.sa = J.so = s.par.sg;
+    J.sb = s.par.sh;
+    J.f0 = J.old = s.par.g + fx_at(xp);
+    J.f1 = s.par.h + fx_at(xp);
+    J.end = kChild;
+    J.neg = s.psign < 0;
+    J.dst = s.src.g + fx_at(s.psign == 0 ? 2 * x : xs + x);
+    if (s.psign == 0) J.twin = s.src.g + fx_at(2 * x + 1);
+    J.sd = s.src.sg;
   } else {
-    const int P = tree_polys(M);
+    const int M = s.M, r = 2 * M, P = tree_polys(M);
     const int col_a = (r - 2) * (r - 3) / 2, col_b = (r - 1) * (r - 2) / 2, col_v = r * (r - 1) / 2;
-    stride = ld * P;
-    const int nA = nmain - q;  // phase step
+    J.sa = J.sb = J.so = s.src.sA;
+    const int nA = s.nmain - s.src.q;  // phase step
     if (s.kind == kTreeLast1) {
-      const int x = it / 6, p = it - 6 * x;
+      const int x = tree_div(it, 6, s.inv_node), p = it - 6 * x, at = (xs + x) * P;
       int j, k;
       tree_pair(p, j, k);
-      const Fxc* A = s.src.A + (ptrdiff_t)x * P;
-      f0 = A + 6 + j;
-      f1 = A + 6 + k;
-      end = kStore;
-      old = A + p;
-      dst = s.src.h + (ptrdiff_t)x * 8 + p;
-      dstride = ld * 8;
-      extra = p == 0 ? 6 : (p == 5 ? 2 : 0);
+      J.f0 = fx_at(at + 6 + j);
+      J.f1 = fx_at(at + 6 + k);
+      J.end = kStore;
+      J.old = fx_at(at + p);
+      const int w = 8 * (xs + x);
+      J.dst = s.src.h + fx_at(w + p);
+      J.sd = s.src.sh;
+      if (p == 0) J.twin = s.src.h + fx_at(w + 6);
+      if (p == 5) J.twin = s.src.h + fx_at(w + 7);
+      J.neg = p == 0;
     } else if (it < nA) {
       const int Pc = tree_polys(M - 1), rc = r - 2, loop0 = rc * (rc - 1) / 2;
-      const int x = it / Pc, p = it - x * Pc;
-      const Fxc* A = s.src.A + (ptrdiff_t)x * P;
-      int j, k;
+      const int x = tree_div(it, Pc, s.inv_node), p = it - x * Pc, at = (xs + x) * P;
+      int j, ka, kb, o = p;
       if (p >= loop0) {  // v'_j
         j = p - loop0;
-        f1 = A + col_v + r - 1;
-        f3 = A + col_v + r - 2;
-        old = A + col_v + j;
+        ka = col_v + r - 2;
+        kb = col_v + r - 1;
+        o = col_v + j;
       } else {
+        int k;
         tree_pair(p, j, k);
-        f1 = A + col_b + k;
-        f3 = A + col_a + k;
-        old = A + p;
+        ka = col_a + k;
+        kb = col_b + k;
       }
-      f0 = A + col_a + j;
-      f2 = A + col_b + j;
-      end = kChild;
-      twin = s.single ? 0 : Pc;
-      dst = s.dst.A + (ptrdiff_t)(s.single ? x : 2 * x) * Pc + p;
-      dstride = s.dst.ld * Pc;
+      J.f0 = fx_at(at + col_a + j);
+      J.f1 = fx_at(at + kb);
+      J.g0 = fx_at(at + col_b + j);
+      J.g1 = fx_at(at + ka);
+      J.old = fx_at(at + o);
+      J.end = kChild;
+      J.db = s.dst.A;
+      const int c = (s.single ? x : 2 * x) * Pc + p;  // the children's storage starts at node 0
+      J.dst = fx_at(c);
+      if (!s.single) J.twin = fx_at(c + Pc);
+      J.sd = s.dst.sA;
     } else {  // h = A_ab + v_a v_b
-      const int x = it - nA;
-      const Fxc* A = s.src.A + (ptrdiff_t)x * P;
-      f0 = A + col_v + r - 2;
-      f1 = A + col_v + r - 1;
-      end = kStore;
-      old = A + col_b + r - 2;
-      dst = s.src.h + x;
-      dstride = ld;
+      const int x = it - nA, at = (xs + x) * P;
+      J.f0 = fx_at(at + col_v + r - 2);
+      J.f1 = fx_at(at + col_v + r - 1);
+      J.end = kStore;
+      J.old = fx_at(at + col_b + r - 2);
+      J.dst = s.src.h + fx_at(xs + x);
+      J.sd = s.src.sh;
     }
-    ostride = stride;
   }
-  FxAcc acc0 = fx_acc_zero(), acc1 = fx_acc_zero();
+  return J;
+}
+
+// What becomes of coefficient t of the product.
+GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& bad) {
+  if (J.end == kChild) {
+    Fxc o{};
+    if (t < J.last) o = fx_load(J.fb + J.old + (ptrdiff_t)(t + 1) * J.so);
+    char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
+    if (!J.neg) fx_store(d + J.dst, fx_add(o, v, bad));
+    if (J.twin >= 0 || J.neg) fx_store(d + (J.neg ? J.dst : J.twin), fx_sub(o, v, bad));
+    if (t == 0) {
+      const Fxc c = fx_load(J.fb + J.old);
+      fx_store(J.db + J.dst, c);
+      if (J.twin >= 0) fx_store(J.db + J.twin, c);
+    }
+  } else {
+    char* d = J.db + (ptrdiff_t)t * J.sd;
+    fx_store(d + J.dst, fx_add(fx_load(J.fb + J.old + (ptrdiff_t)t * J.so), v, bad));
+    if (J.twin >= 0) {
+      const Fxc zero{};
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, bad), v, bad) : v);
+    }
+  }
+}
+
+// The same in four independent parts, and the number that a part starts from.
+GBSH_HD Fxc tree_end_old(const TreeJob& J, int t, int role) {
+  if (J.end == kDot) return role == 0 ? fx_load(J.fb + J.old + (ptrdiff_t)(J.last - t) * J.so) : Fxc{};
+  if (J.end == kStore) return role == 0 ? fx_load(J.fb + J.old + (ptrdiff_t)t * J.so) : Fxc{};
+  if (role < 2) return t < J.last ? fx_load(J.fb + J.old + (ptrdiff_t)(t + 1) * J.so) : Fxc{};
+  return t == 0 ? fx_load(J.fb + J.old) : Fxc{};
+}
+GBSH_HD void tree_end_part(const TreeJob& J, int t, int role, const Fxc& o, const Fxc& v, unsigned& bad) {
+  if (J.end == kStore) {
+    char* d = J.db + (ptrdiff_t)t * J.sd;
+    if (role == 0) {
+      fx_store(d + J.dst, fx_add(o, v, bad));
+    } else if (role == 1 && J.twin >= 0) {
+      const Fxc zero{};
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, bad), v, bad) : v);
+    }
+    return;
+  }
+  char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
+  if (role < 2) {
+    if (role == 1 && J.twin < 0) return;
+    if (role == 0 && !J.neg) fx_store(d + J.dst, fx_add(o, v, bad));
+    else fx_store(d + (role == 0 ? J.dst : J.twin), fx_sub(o, v, bad));
+  } else if (t == 0 && (role == 2 || J.twin >= 0)) {
+    fx_store(J.db + (role == 2 ? J.dst : J.twin), o);
+  }
+}
+
+// A task's work in pieces for phases with few items: piece `sub` (of four) of coefficient t of
+// item `it`, a quarter of its products. The four sums are added (by the caller: exactly, they are
+// integers) before tree_end_part.
+GBSH_HD FxAcc tree_piece(const TreeJob& J, int t, int sub) {
+  FxAcc acc{0, 0, 0, 0, 0, 0};
+  if (sub == 0) acc = fx_acc_zero();
+  if (t > J.top + 1) return acc;
+  const bool two = J.g0 >= 0;
+  const int u0 = two ? sub >> 1 : sub, du = two ? 2 : 4;
+  const char* a = J.fb + (two && (sub & 1) ? J.g0 : J.f0) + (ptrdiff_t)u0 * J.sa;
+  const char* b = J.fb + (two && (sub & 1) ? J.g1 : J.f1) + (ptrdiff_t)(t - u0) * J.sb;
+#ifdef __CUDA_ARCH__
+#pragma unroll 4
+#endif
+  for (int u = u0; u <= t; u += du) {
+    fx_mac(acc, fx_load(a), fx_load(b));
+    a += (ptrdiff_t)du * J.sa;
+    b -= (ptrdiff_t)du * J.sb;
+  }
+  return acc;
+}
+GBSH_HD int tree_pieces(const TreePhase& s) { return (s.n - s.M + 1) * s.items * 4; }
+
+// Runs one task of walk `walk`. In phase last2 returns true with a part of node `node`'s term in
+// z (sums of limbs, carries not propagated).
+GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, int& node, Fxc& z, unsigned& bad) {
+  const int L = s.n - s.M + 1, tiles = (L + 1) / 2;
+  int tile = tree_div(task, s.items, s.inv_items);
+  const TreeJob J = tree_job(s, walk, task - tile * s.items);
+  node = J.node;
+  z = Fxc{};
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
-  for (;;) {
-    fx_conv2(acc0, acc1, f0, stride, f1, stride, t0);
-    if (!f2) break;
-    f0 = f2;
-    f1 = f3;
-    f2 = nullptr;
-  }
-  FxAcc dot = fx_acc_zero();
+  for (int side = 0;; ++side) {
+    const int t0 = J.top - 2 * tile;
+    if (t0 >= -1) {
+      FxAcc acc0 = fx_acc_zero(), acc1 = fx_acc_zero();
+      int a = J.f0, b = J.f1;
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
-  for (int t = t0; t < t0 + 2; ++t) {
-    const Fxc v = fx_norm(acc0, bad);
-    acc0 = acc1;
-    if (t < 0) continue;
-    if (end == kChild) {
-      Fxc o{};
-      if (t + 1 < Lold) o = fx_load(old + (ptrdiff_t)(t + 1) * ostride);
-      Fxc* d = dst + (ptrdiff_t)(t + 1) * dstride;
-      fx_store(d, fx_add(o, v, twin ? 1 : sg, bad));
-      if (twin) fx_store(d + twin, fx_add(o, v, -1, bad));
-      if (t == 0) {
-        const Fxc c = fx_load(old);
-        fx_store(dst, c);
-        if (twin) fx_store(dst + twin, c);
+      for (bool more = J.g0 >= 0;; more = false) {
+        fx_conv2(acc0, acc1, J.fb + a, J.sa, J.fb + b, J.sb, t0);
+        if (!more) break;
+        a = J.g0;
+        b = J.g1;
       }
-    } else if (end == kStore) {
-      Fxc* d = dst + (ptrdiff_t)t * dstride;
-      fx_store(d, fx_add(fx_load(old + (ptrdiff_t)t * ostride), v, 1, bad));
-      if (extra == 2) fx_store(d + extra, v);
-      if (extra == 6) {
-        const Fxc zero{};
-        fx_store(d + extra, fx_add(fx_add(zero, v, -1, bad), v, -1, bad));
+#ifdef __CUDA_ARCH__
+#pragma unroll 1
+#endif
+      for (int t = t0; t < t0 + 2; ++t) {
+        const Fxc v = fx_norm(acc0, bad);
+        acc0 = acc1;
+        if (t < 0) continue;
+        if (J.end == kDot) {
+          FxAcc dot = fx_acc_zero();
+          fx_mac(dot, v, fx_load(J.fb + J.old + (ptrdiff_t)(L - 1 - t) * J.so));
+          const Fxc part = fx_norm(dot, bad);
+          z = Fxc{z.rh + part.rh, z.rm + part.rm, z.rl + part.rl, z.ih + part.ih, z.im + part.im, z.il + part.il};
+        } else {
+          tree_end(J, t, v, bad);
+        }
       }
-    } else {
-      fx_mac(dot, v, fx_load(old + (ptrdiff_t)(L - 1 - t) * ostride));
     }
+    const int mirror = tiles - 1 - tile;
+    if (side == 1 || mirror == tile) break;
+    tile = mirror;
   }
-  if (end != kDot) return false;
-  z = fx_norm(dot, bad);
-  return true;
+  return J.end == kDot;
 }
 
 // ------------------------------------------------------------------ cutting the tree
-// Step `step` of the breadth-first part (level n - step to n - step - 1) of a tree whose levels
-// n, n - 1, ... follow each other from `base`.
-GBSH_HD TreePhase tree_step_phase(Fxc* base, int n, int step) {
+// Phase i of n of the whole tree breadth first; its levels n, n - 1, ... follow each other from
+// `base`.
+GBSH_HD TreePhase tree_whole_phase(char* base, int n, int i) {
   TreePhase s;
-  const int M = n - step;
-  s.kind = kTreeStep;
+  const int M = n - i > 2 ? n - i : 2;
+  const int up = M < n ? M + 1 : M, down = M > 2 ? M - 1 : 2;
+  s.src = tree_level(base + tree_offset(M, n), M, n, tree_width(M, n));
+  s.dst = tree_level(base + tree_offset(down, n), down, n, tree_width(down, n));
+  s.par = tree_level(base + tree_offset(up, n), up, n, tree_width(up, n));
+  s.kind = i < n - 2 ? kTreeStep : (i == n - 2 ? kTreeLast1 : kTreeLast2);
   s.n = n;
   s.M = M;
-  s.src = tree_level(base + tree_offset(M, n), M, n, tree_width(M, n));
-  s.dst = tree_level(base + tree_offset(M - 1, n), M - 1, n, tree_width(M - 1, n));
-  s.par = s.src;
-  if (step > 0) s.par = tree_level(base + tree_offset(M + 1, n), M + 1, n, tree_width(M + 1, n));
-  s.single = step == 0;
-  s.psign = step == 1 ? 1 : 0;
-  s.gsel = 0;
+  s.single = i == 0 && n > 2;
+  s.psign = M == n - 1 ? 1 : 0;
+  s.src_bit = s.par_bit = -1;
+  tree_ready(s);
   return s;
 }
 
-// A unit: node `unit` of level m1 and all below it, in scratch of tree_scratch elements. Levels
+// A unit: node `unit` of level m1 and all below it, in scratch of tree_scratch bytes. Levels
 // m1 - 1 .. top are walked depth first and hold the two children of one node each; from level
 // `top` on the subtree is worked off breadth first.
 GBSH_HD size_t tree_scratch(int n, int m1, int top) {
   size_t e = 0;
-  for (int M = m1 - 1; M >= 2; --M) e += tree_level_elems(M, n, M >= top ? 2 : 1 << (top - M));
+  for (int M = m1 - 1; M >= 2; --M) e += tree_level_bytes(M, n, M >= top ? 2 : 1 << (top - M));
   return e;
 }
-GBSH_HD void tree_unit_levels(TreeLevel* lv, Fxc* base, Fxc* scratch, int n, int m1, int top, int unit) {
-  lv[m1] = tree_node(tree_level(base + tree_offset(m1, n), m1, n, tree_width(m1, n)), m1, unit);
+GBSH_HD void tree_unit_levels(TreeLevel* lv, char* base, char* scratch, int n, int m1, int top, int unit) {
+  lv[m1] = tree_node(tree_level(base + tree_offset(m1, n), m1, n, tree_width(m1, n)), unit);
   if (m1 < n)
-    lv[m1 + 1] = tree_node(tree_level(base + tree_offset(m1 + 1, n), m1 + 1, n, tree_width(m1 + 1, n)),
-                           m1 + 1, unit >> 1);
+    lv[m1 + 1] = tree_node(tree_level(base + tree_offset(m1 + 1, n), m1 + 1, n, tree_width(m1 + 1, n)), unit >> 1);
   for (int M = m1 - 1; M >= 2; --M) {
     const int q = M >= top ? 2 : 1 << (top - M);
     lv[M] = tree_level(scratch, M, n, q);
-    scratch += tree_level_elems(M, n, q);
+    scratch += tree_level_bytes(M, n, q);
   }
 }
-// Phase i (of m1) of walk b (of 2^(m1 - top)). Bit M - top of b tells which child of level M
-// the walk is in. Walk b > 0 shares with walk b - 1 the levels above the one whose child
-// changes, so it starts at phase tree_first_phase.
+// The unit is worked off in walks b = 0 .. 2^(m1 - top) - 1 of m1 phases each. Bit M - top of b
+// tells which child of level M the walk is in. Walk b > 0 shares with walk b - 1 the levels above
+// the one whose child changes, so it starts at phase tree_first_phase.
 GBSH_HD int tree_first_phase(int m1, int top, unsigned b) {
   if (b == 0) return 0;
   int low = 0;
   while (!((b >> low) & 1)) ++low;
   return m1 - top - low;
 }
-GBSH_HD TreePhase tree_unit_phase(const TreeLevel* lv, int n, int m1, int top, int unit, unsigned b, int i) {
+GBSH_HD TreePhase tree_unit_phase(const TreeLevel* lv, int n, int m1, int top, int unit, int i) {
   TreePhase s;
   const int M = m1 - i > 2 ? m1 - i : 2;
   s.n = n;
@@ -480,13 +602,17 @@ GBSH_HD TreePhase tree_unit_phase(const TreeLevel* lv, int n, int m1, int top, i
   s.dst = lv[M > 2 ? M - 1 : 2];
   s.par = lv[M < n ? M + 1 : M];
   s.psign = 0;
-  s.gsel = 0;
+  s.src_bit = s.par_bit = -1;
   if (M < m1 && M >= top) {
-    s.gsel = (b >> (M - top)) & 1;
-    s.src = tree_node(s.src, M, s.gsel);
+    s.src_bit = M - top;
+    s.src.q = 1;
   }
-  if (M + 1 < m1 && M + 1 >= top) s.par = tree_node(s.par, M + 1, (b >> (M + 1 - top)) & 1);
+  if (M + 1 < m1 && M + 1 >= top) {
+    s.par_bit = M + 1 - top;
+    s.par.q = 1;
+  }
   if (M == m1) s.psign = m1 < n - 1 && (unit & 1) ? -1 : 1;
+  tree_ready(s);
   return s;
 }
 

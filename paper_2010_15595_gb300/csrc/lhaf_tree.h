@@ -11,15 +11,15 @@
 
 namespace gbsh {
 
-// One problem of a launch. Its levels n .. m1 are computed breadth first by the whole GPU; each
-// node of level m1 is a unit that one CTA works off: depth first, two nodes a level, down to
-// level `top`, then breadth first.
+// One problem of a launch. A small one is worked off whole by a cluster of CTAs. Of the others the
+// levels n .. m1 are computed breadth first by the whole GPU; each node of level m1 is a unit that
+// one CTA works off: depth first, two nodes a level, down to level `top`, then breadth first.
 struct TreeProblem {
   BatchInput in;
   int Ne, n;       // padded size, Ne = 2 n >= 4
   int m1, top;
   unsigned unit_base, units;
-  size_t root;     // element offset of its levels n .. m1
+  size_t root;     // byte offset of its levels n .. m1
 };
 
 // Running state of a problem: exact limb sums of the signed mean, and how to undo the scale.
@@ -36,12 +36,16 @@ struct TreeState {
 struct TreePlan {
   std::vector<TreeProblem> prob;   // in launch order
   std::vector<int> order;          // prob[q] is the caller's problem order[q]
+  int nbig;                        // prob[0 .. nbig) are large, the others small
+  int cluster, clusters;           // CTAs per cluster and clusters of the small ones' launch
+  size_t small_bytes;              // scratch per cluster
   unsigned total_units;
+  int fine;                        // breadth-first steps of at most so many pieces run in pieces
   int blocks;
-  struct Step { int problems; unsigned tasks; };
+  struct Step { int problems; int tasks; };
   std::vector<Step> steps;         // breadth-first eliminations: problems that take part (the
                                    // first ones), most tasks of one of them
-  size_t cta_elems;                // scratch elements per CTA
+  size_t cta_bytes;                // scratch per CTA
   size_t off_prob, off_state, off_counter, off_out, off_root, off_cta, bytes;
 };
 
@@ -56,6 +60,11 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
 
 // Fills in the inputs and, for more than one problem, uploads the table.
 cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st);
+
+// Stages and launches `plan`, waits, and copies the results to out3[3 i ..] of the caller's
+// problem i (re, im, 0); problems to be evaluated by the subset sum are added to `again`.
+cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st, double* out3,
+                     std::vector<int>* again);
 
 // Device address of a one-problem launch's fallback flag (nonzero: evaluate by the subset sum).
 const unsigned* tree_flag(const TreePlan& plan, void* ws);

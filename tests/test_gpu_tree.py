@@ -26,32 +26,54 @@ def _async(gbsh, A, prec, nbytes=None):
     return complex(out.item())
 
 
-# 1..6: padding to four vertices, no signed pair, one signed pair; 13..16 and 19, 20: units
-# above and at the breadth-first level; 23: odd
-@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6, 7, 8, 13, 14, 16, 19, 20, 23])
+# 1..6: padding to four vertices, no signed pair, one signed pair; 8, 10, 12, 16, 18: cluster
+# sizes of the small kernel; 24, 25, 26: its last size and the first ones of the other kernels
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 13, 16, 18, 19, 23, 24, 25, 26])
 def test_sizes_and_entry_points(gbsh, N):
     rng = np.random.default_rng(700 + N)
     for A in (W.single_lhaf_mid(N), W.random_complex_symmetric(N, rng)):
-        ref = L.lhaf_brute(A) if N <= 12 else L.lhaf_dp(A)
+        tol = TOL
+        if N <= 24:
+            ref = L.lhaf_brute(A) if N <= 12 else L.lhaf_dp(A)
+        else:  # the long-double subset sum and its own rounding floor
+            ref = L.lhaf_subset_ld(A)
+            tol = max(TOL, 512 * 2.0 ** -64 * L.lhaf_subset_stats(A)[2] ** 0.5 / abs(ref))
         got = gbsh.lhaf(A, precision=gbsh.PREC_TF)
-        assert abs(got - ref) <= TOL * abs(ref), (N, got, ref)
+        assert abs(got - ref) <= tol * abs(ref), (N, got, ref)
         assert gbsh.lhaf(_dev(A), precision=gbsh.PREC_TF) == got
         assert _async(gbsh, A, gbsh.PREC_TF) == got
         big = np.zeros((N, N + 3), complex)
         big[:, :N] = A
         assert gbsh.lhaf(_dev(big)[:, :N], precision=gbsh.PREC_TF) == got  # leading dimension
+        if N <= 24:  # FP64 entry points: the same evaluation
+            assert gbsh.lhaf(A) == got and _async(gbsh, A, gbsh.PREC_FP64) == got
+            B = np.zeros((N + 2, N + 2), complex)
+            B[:N, :N] = A
+            g = np.concatenate([np.diag(A), [3, 4]])
+            pattern = [1] * N + [0, 0]
+            assert gbsh.gbs_prob(B, g, pattern, return_lhaf=True)[1] == got
+            assert gbsh.gbs_prob_batch(B, g, [pattern, pattern])[1][1] == got
 
 
 def test_batch_equals_single(gbsh):
-    """Every size 0..31 in one batch and alone: the limb sums are exact, so the bits agree."""
+    """Every size 0..31 in one batch and alone, a batch of small problems large enough for
+    one-CTA clusters, and a mixed-precision one: the limb sums are exact, so the bits agree."""
     rng = np.random.default_rng(71)
     mats = [W.random_complex_symmetric(N, rng) for N in list(range(32)) + [7, 7, 30, 1]]
-    got = gbsh.lhaf_batch(mats, precision=gbsh.PREC_TF)
-    for A, g in zip(mats, got):
-        if A.shape[0] == 0:
-            assert g == 1
-        else:
-            assert g == gbsh.lhaf(A, precision=gbsh.PREC_TF), A.shape
+    many = [W.random_complex_symmetric(1 + i % 18, rng) for i in range(330)]
+    for batch in (mats, many, mats[:25]):
+        got = gbsh.lhaf_batch(batch, precision=gbsh.PREC_TF)
+        for A, g in zip(batch, got):
+            if A.shape[0] == 0:
+                assert g == 1
+            else:
+                assert g == gbsh.lhaf(A, precision=gbsh.PREC_TF), A.shape
+    fp64 = gbsh.lhaf_batch(mats)
+    mixed = gbsh.lhaf_batch(mats, precision=gbsh.PREC_MIXED)
+    tf = gbsh.lhaf_batch(mats, precision=gbsh.PREC_TF)
+    for i in range(25):  # N <= 24
+        assert fp64[i] == tf[i]
+        assert mixed[i] == fp64[i] if i > gbsh.C32_MAX_N else abs(mixed[i] - fp64[i]) <= 1e-5 * abs(fp64[i])
 
 
 @pytest.mark.parametrize("N", [6, 11, 20])
@@ -80,16 +102,19 @@ def test_handed_back_to_the_subset_sum(gbsh, N):
 
 def test_workspace_of_the_subset_sum_is_still_taken(gbsh):
     """A workspace too small for the tree but large enough for the subset sum is accepted."""
-    A = W.single_lhaf_mid(18)
-    small = gbsh.workspace_size(18)  # the FP64 subset sum's, which the triple-float one fits too
-    v = _async(gbsh, A, gbsh.PREC_TF, nbytes=max(small, 1 << 16))
-    assert abs(v - gbsh.lhaf(A, precision=gbsh.PREC_TF)) <= 1e-13 * abs(v)
+    A = W.single_lhaf_mid(24)
+    small = gbsh.workspace_size(26)  # FP64 above N = 24: the subset sum's alone, larger than N = 24's
+    assert small < gbsh.workspace_size(24, gbsh.PREC_TF)
+    for prec in (gbsh.PREC_FP64, gbsh.PREC_TF):
+        v = _async(gbsh, A, prec, nbytes=small)
+        subset, _ = gbsh.lhaf(A, precision=prec, return_error=True)
+        assert v == subset
 
 
 def test_graph_capture(gbsh):
     """lhaf_async inside a CUDA graph: replays read the matrix that is there at replay time."""
     import torch
-    N = 20
+    N = 26
     A, B = W.single_lhaf_mid(N), W.single_lhaf_mid(N, seed=1)
     dA = _dev(A)
     out = torch.zeros(1, dtype=torch.complex128, device="cuda")

@@ -17,34 +17,35 @@ void to_fixed(double x, int m, int e, int& h, int& mm, int& l) {  // x m 2^e
   if (sh >= 0) v <<= sh;
   else if (sh < -100) v = 0;
   else v = (v + ((__int128)1 << (-sh - 1))) >> (-sh);
-  l = sext28((long long)v);
-  v = (v - l) >> kLimbBits;
-  mm = sext28((long long)v);
-  v = (v - mm) >> kLimbBits;
-  h = (int)v;
+  v += kLimbHalf;
+  l = ((int)(long long)v & kLimbMask) - kLimbHalf;
+  v = (v >> kLimbBits) + kLimbHalf;
+  mm = ((int)(long long)v & kLimbMask) - kLimbHalf;
+  h = (int)(long long)(v >> kLimbBits);
 }
 
-// Guarded storage: a level's elements and a canary on each side.
+// Guarded storage: a buffer with a canary on each side.
 struct Guarded {
-  std::vector<Fxc> mem;
-  explicit Guarded(size_t n) : mem(n + 64, Fxc{7, 7, 7, 7, 7, 7, 7, 7}) {}
-  Fxc* data() { return mem.data() + 32; }
+  std::vector<char> mem;
+  explicit Guarded(size_t n) : mem(n + 2048, 7) {}
+  char* data() { return mem.data() + 1024; }
   bool intact() const {
-    for (int i = 0; i < 32; ++i)
-      if (mem[i].rh != 7 || mem[mem.size() - 1 - i].rh != 7 || mem[i].il != 7 || mem[mem.size() - 1 - i].il != 7)
-        return false;
+    for (int i = 0; i < 1024; ++i)
+      if (mem[i] != 7 || mem[mem.size() - 1 - i] != 7) return false;
     return true;
   }
 };
 }  // namespace
 
+// (level m1 = 0: the whole tree breadth first.)
 // lhaf of the N x N row-major complex matrix a (re, im pairs) whose vertices are scaled by
 // m / 16 2^e; units are the nodes of level m1, breadth first from level top. Returns 0, or 1 on
 // overflow, 2 on a write outside a buffer.
 extern "C" int tree_host_lhaf(const double* a, int N, int m, int e, int m1, int top, double* out) {
   const int Ne = std::max(4, N + (N & 1)), n = Ne / 2;
-  Guarded levels(tree_offset(m1 - 1, n)), scratch(tree_scratch(n, m1, top));
-  Fxc* root = levels.data();
+  const bool whole = m1 == 0;
+  Guarded levels(tree_offset(whole ? 1 : m1 - 1, n)), scratch(whole ? 0 : tree_scratch(n, m1, top));
+  const TreeLevel root = tree_level(levels.data(), n, n, 1);
   const int edges = Ne * (Ne - 1) / 2;
   for (int p = 0; p < tree_polys(n); ++p) {
     int j, k;
@@ -58,33 +59,39 @@ extern "C" int tree_host_lhaf(const double* a, int N, int m, int e, int m1, int 
     } else if (j == k) {
       v.rh = 1 << (kTreeFrac - 1 - 2 * kLimbBits);
     }
-    fx_store(root + p, v);
+    fx_store(root.A + fx_at(p), v);
   }
   Fxc one{};
   one.rh = 1 << (kTreeFrac - 2 * kLimbBits);
-  fx_store(root + tree_polys(n), one);
+  fx_store(root.A + root.g, one);
   unsigned bad = 0;
   int node;
   Fxc z;
-  for (int step = 0; n - step > m1; ++step) {
-    const TreePhase s = tree_step_phase(root, n, step);
-    for (unsigned t = 0; t < tree_tasks(s); ++t) tree_task(s, t, node, z, bad);
-  }
   __int128 re = 0, im = 0;
-  for (int unit = 0; unit < tree_width(m1, n); ++unit) {
+  auto add = [&](bool neg) {
+    const __int128 x = (((__int128)z.rh << kLimbBits) + z.rm) * (1 << kLimbBits) + z.rl;
+    const __int128 y = (((__int128)z.ih << kLimbBits) + z.im) * (1 << kLimbBits) + z.il;
+    re += neg ? -x : x;
+    im += neg ? -y : y;
+  };
+  for (int i = 0; whole && i < n; ++i) {
+    const TreePhase s = tree_whole_phase(levels.data(), n, i);
+    for (int t = 0; t < s.tasks; ++t)
+      if (tree_task(s, 0, t, node, z, bad)) add(__builtin_popcount(node) & 1);
+  }
+  for (int step = 0; !whole && n - step > m1; ++step) {
+    const TreePhase s = tree_whole_phase(levels.data(), n, step);
+    for (int t = 0; t < s.tasks; ++t) tree_task(s, 0, t, node, z, bad);
+  }
+  for (int unit = 0; !whole && unit < tree_width(m1, n); ++unit) {
     TreeLevel lv[34];
-    tree_unit_levels(lv, root, scratch.data(), n, m1, top, unit);
+    tree_unit_levels(lv, levels.data(), scratch.data(), n, m1, top, unit);
     for (unsigned b = 0; b < 1u << (m1 - top); ++b)
       for (int i = tree_first_phase(m1, top, b); i < m1; ++i) {
-        const TreePhase s = tree_unit_phase(lv, n, m1, top, unit, b, i);
-        for (unsigned t = 0; t < tree_tasks(s); ++t)
-          if (tree_task(s, t, node, z, bad)) {
-            const bool neg = (__builtin_popcount(node) + __builtin_popcount(unit) + __builtin_popcount(b)) & 1;
-            const __int128 x = (((__int128)z.rh << 28) + z.rm) * (1 << 28) + z.rl;
-            const __int128 y = (((__int128)z.ih << 28) + z.im) * (1 << 28) + z.il;
-            re += neg ? -x : x;
-            im += neg ? -y : y;
-          }
+        const TreePhase s = tree_unit_phase(lv, n, m1, top, unit, i);
+        for (int t = 0; t < s.tasks; ++t)
+          if (tree_task(s, b, t, node, z, bad))
+            add((__builtin_popcount(node) + __builtin_popcount(unit) + __builtin_popcount(b)) & 1);
       }
   }
   const int exp2 = -kTreeFrac - (n >= 3 ? n - 3 : 0) - e * N + (Ne - N);
