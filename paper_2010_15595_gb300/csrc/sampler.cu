@@ -36,6 +36,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <numeric>
 #include <thread>
 #include <vector>
 
@@ -44,6 +45,7 @@
 #include "../../include/gbsh.h"
 #include "batch_host.h"
 #include "lhaf_kernels.cuh"
+#include "lhaf_tree.h"
 
 namespace {
 
@@ -381,26 +383,71 @@ int gbsh_sampler::tick(std::vector<Chain>& active) {
     in[q] = gbsh::BatchInput{dB, dgam + (size_t)active[cands[q].chain].slot * M,
                              didx + cands[q].idx_off, M, cands[q].N};
   }
-  if (cfg.batching) {
-    if (nc > 0) {
-      gbsh::BatchLayout L = gbsh::batch_layout(Ns.data(), nc, 0);
-      rc = ensure_ws(L.bytes);
-      if (rc != GBSH_OK) return rc;
-      e = gbsh::batch_run(L, in, nc, cfg.precision, 0, ws, st, out3.data());
+  // FP64 loop hafnians of the candidates by the elimination tree (lhaf_tree.cuh; sums of exact
+  // integers, so a candidate's value is the same alone and in any mix); the complex-FP32 variant,
+  // and what the tree hands back, by the subset sum.
+  std::vector<int> rest;
+  if (cfg.precision == GBSH_PREC_FP64) {
+    std::vector<int> sel, n;
+    for (int q = 0; q < nc; ++q) {
+      if (Ns[q] > 0) {
+        sel.push_back(q);
+        n.push_back(Ns[q]);
+      } else {
+        out3[3 * (size_t)q] = 1.0;
+      }
+    }
+    // batching: all candidates in one launch; plain path: one launch sequence and one
+    // synchronisation per candidate, what a caller of gbsh_gbs_prob would do
+    const size_t step = cfg.batching ? std::max<size_t>(sel.size(), 1) : 1;
+    for (size_t f = 0; f < sel.size(); f += step) {
+      const size_t m = std::min(step, sel.size() - f);
+      gbsh::TreePlan T;
+      e = gbsh::tree_plan(n.data() + f, (int)m, 0, &T);
       if (e != cudaSuccess) return from_cuda(e);
+      rc = ensure_ws(T.bytes);
+      if (rc != GBSH_OK) return rc;
+      std::vector<gbsh::BatchInput> some(m);
+      for (size_t q = 0; q < m; ++q) some[q] = in[sel[f + q]];
+      std::vector<double> o(3 * m);
+      std::vector<int> again;
+      e = gbsh::tree_run(&T, some.data(), ws, st, o.data(), &again);
+      if (e != cudaSuccess) return from_cuda(e);
+      for (size_t q = 0; q < m; ++q)
+        for (int j = 0; j < 3; ++j) out3[3 * (size_t)sel[f + q] + j] = o[3 * q + j];
+      for (int q : again) rest.push_back(sel[f + q]);
     }
   } else {
-    // plain path: one single-evaluation launch sequence (expansion of B, the fill vector and
-    // the pattern on the device, the popcount-class launches, finalize) and one
-    // synchronisation per loop hafnian -- what a caller of gbsh_gbs_prob would do per
-    // candidate. The complex-FP32 and double-double variants exist only in the batched
+    rest.resize(nc);
+    std::iota(rest.begin(), rest.end(), 0);
+  }
+  if (cfg.batching) {
+    if (!rest.empty()) {
+      std::vector<int> n(rest.size());
+      std::vector<gbsh::BatchInput> some(rest.size());
+      for (size_t q = 0; q < rest.size(); ++q) {
+        n[q] = Ns[rest[q]];
+        some[q] = in[rest[q]];
+      }
+      std::vector<double> o(3 * rest.size());
+      gbsh::BatchLayout L = gbsh::batch_layout(n.data(), (int)rest.size(), 0);
+      rc = ensure_ws(L.bytes);
+      if (rc != GBSH_OK) return rc;
+      e = gbsh::batch_run(L, some, (int)rest.size(), cfg.precision, 0, ws, st, o.data());
+      if (e != cudaSuccess) return from_cuda(e);
+      for (size_t q = 0; q < rest.size(); ++q)
+        for (int j = 0; j < 3; ++j) out3[3 * (size_t)rest[q] + j] = o[3 * q + j];
+    }
+  } else {
+    // plain path, subset sum: one single-evaluation launch sequence and one synchronisation per
+    // loop hafnian. The complex-FP32 and double-double variants exist only in the batched
     // kernel, so for them each candidate is a one-problem batch instead.
     gbsh::DeviceInfo dev;
     e = gbsh::device_info(&dev);
     if (e != cudaSuccess) return from_cuda(e);
     e = gbsh::ensure_constants();
     if (e != cudaSuccess) return from_cuda(e);
-    for (int q = 0; q < nc; ++q) {
+    for (int q : rest) {
       if (Ns[q] == 0) {
         out3[3 * (size_t)q] = 1.0;
         out3[3 * (size_t)q + 1] = 0.0;
