@@ -318,7 +318,7 @@ __device__ __forceinline__ TreeJob tree_piece_job(const TreePhase& s, int id, in
 }
 __device__ __forceinline__ bool tree_piece_task(const TreeJob& J, int t, int sub, Fxc& z, unsigned& bad) {
   const bool active = t <= J.top + 1;
-  FxAcc acc{0, 0, 0, 0, 0, 0};
+  FxSum acc{0, 0, 0, 0, 0, 0};
   Fxc old{};
   if (active) {
     old = tree_end_old(J, t, sub);
@@ -342,9 +342,18 @@ __device__ __forceinline__ bool tree_piece_task(const TreeJob& J, int t, int sub
   if (sub != 0) return false;
   FxAcc dot = fx_acc_zero();
   fx_mac(dot, v, old);
-  z = fx_norm(dot, bad);
+  z = fx_norm(fx_sum(dot), bad);
   return true;
 }
+
+// Column of a thread in its CTA's job storage (tree_put). Volatile: the compiler would keep the
+// values in registers, and spill those of the products instead.
+template <int kThreads>
+struct JobSlot {
+  volatile int (*m)[kThreads];
+  __device__ __forceinline__ void put(int k, int v) const { m[k][threadIdx.x] = v; }
+  __device__ __forceinline__ int get(int k) const { return m[k][threadIdx.x]; }
+};
 
 // kOne: the phase of the one problem is set up on the host. Phases of at most `fine` pieces run in
 // pieces.
@@ -353,6 +362,7 @@ __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ TreePhase one, int step, int fine,
                  TreeState* __restrict__ state, char* __restrict__ levels) {
   __shared__ TreePhase many;
+  __shared__ int slots[kSlotInts][kTreeThreads];
   if (!kOne) {
     if (table[blockIdx.y].n - step <= table[blockIdx.y].m1) return;  // fewer steps than another's
     if (threadIdx.x == 0)
@@ -370,7 +380,7 @@ tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ 
       tree_piece_task(J, x, t & 3, z, bad);
     }
   } else if (t < s.tasks) {
-    tree_task(s, 0, t, x, z, bad);
+    tree_task(s, 0, t, JobSlot<kTreeThreads>{slots}, x, z, bad);
   }
   if (bad) atomicOr(&state[blockIdx.y].bad, 1u);
 }
@@ -411,6 +421,7 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
   __shared__ TreeLevel lv[kMaxN / 2 + 2];  // levels m1 + 1 and m1: the unit and its parent
   __shared__ TreePhase phase[kMaxN / 2];
   __shared__ LimbSums<kTreeThreads> sum;
+  __shared__ int slots[kSlotInts][kTreeThreads];
   __shared__ unsigned s_unit;
   __shared__ int s_prob;
   const int tid = threadIdx.x;
@@ -444,7 +455,7 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
         for (int t = tid; t < s.tasks; t += kTreeThreads) {
           int x;
           Fxc z;
-          if (tree_task(s, b, t, x, z, bad))
+          if (tree_task(s, b, t, JobSlot<kTreeThreads>{slots}, x, z, bad))
             sum.add(z, (__popc((unsigned)x) + __popc((unsigned)unit) + __popc(b)) & 1);
         }
         __syncthreads();
@@ -480,6 +491,7 @@ tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int fi
     LimbSums<kRootThreads> sum;
   } sh;
   __shared__ TreePhase phase[kTreeSmallMax];
+  __shared__ int slots[kSlotInts][kRootThreads];
   __shared__ unsigned s_bad;
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), tid = threadIdx.x;
@@ -510,7 +522,7 @@ tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int fi
         }
       } else {
         for (int q = t0; q < s.tasks; q += stride)
-          if (tree_task(s, 0, q, x, z, bad)) sh.sum.add(z, __popc((unsigned)x) & 1);
+          if (tree_task(s, 0, q, JobSlot<kRootThreads>{slots}, x, z, bad)) sh.sum.add(z, __popc((unsigned)x) & 1);
       }
       if (i == P.n - 1) {
         if (bad) atomicOr(&s_bad, 1u);

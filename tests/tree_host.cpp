@@ -24,6 +24,12 @@ void to_fixed(double x, int m, int e, int& h, int& mm, int& l) {  // x m 2^e
   h = (int)(long long)(v >> kLimbBits);
 }
 
+struct HostSlot {
+  int* m;
+  void put(int k, int v) const { m[k] = v; }
+  int get(int k) const { return m[k]; }
+};
+
 // Guarded storage: a buffer with a canary on each side.
 struct Guarded {
   std::vector<char> mem;
@@ -65,7 +71,8 @@ extern "C" int tree_host_lhaf(const double* a, int N, int m, int e, int m1, int 
   one.rh = 1 << (kTreeFrac - 2 * kLimbBits);
   fx_store(root.A + root.g, one);
   unsigned bad = 0;
-  int node;
+  int node, ints[kSlotInts];
+  const HostSlot slot{ints};
   Fxc z;
   __int128 re = 0, im = 0;
   auto add = [&](bool neg) {
@@ -77,11 +84,11 @@ extern "C" int tree_host_lhaf(const double* a, int N, int m, int e, int m1, int 
   for (int i = 0; whole && i < n; ++i) {
     const TreePhase s = tree_whole_phase(levels.data(), n, i);
     for (int t = 0; t < s.tasks; ++t)
-      if (tree_task(s, 0, t, node, z, bad)) add(__builtin_popcount(node) & 1);
+      if (tree_task(s, 0, t, slot, node, z, bad)) add(__builtin_popcount(node) & 1);
   }
   for (int step = 0; !whole && n - step > m1; ++step) {
     const TreePhase s = tree_whole_phase(levels.data(), n, step);
-    for (int t = 0; t < s.tasks; ++t) tree_task(s, 0, t, node, z, bad);
+    for (int t = 0; t < s.tasks; ++t) tree_task(s, 0, t, slot, node, z, bad);
   }
   for (int unit = 0; !whole && unit < tree_width(m1, n); ++unit) {
     TreeLevel lv[34];
@@ -90,7 +97,7 @@ extern "C" int tree_host_lhaf(const double* a, int N, int m, int e, int m1, int 
       for (int i = tree_first_phase(m1, top, b); i < m1; ++i) {
         const TreePhase s = tree_unit_phase(lv, n, m1, top, unit, i);
         for (int t = 0; t < s.tasks; ++t)
-          if (tree_task(s, b, t, node, z, bad))
+          if (tree_task(s, b, t, slot, node, z, bad))
             add((__builtin_popcount(node) + __builtin_popcount(unit) + __builtin_popcount(b)) & 1);
       }
   }
