@@ -29,10 +29,17 @@ namespace {
 
 constexpr int kTreeThreads = 128;
 constexpr int kTreeCtasPerSm = 6;
-// Largest n of a small problem: alone (clusters of up to 16 CTAs), and in a crowd, where a
-// problem gets a CTA or two and its scratch (all levels) must stay in the cache.
-constexpr int kTreeSmallMax = 12;
-constexpr int kTreeSmallCrowd = 8;
+// Largest n of a small problem (tree_small_kernel). Alone, n = 8 takes 53 us that way against 72
+// by launches; n = 9 and 10 the same either way, n = 11 takes 104 against 91 and n = 12 162
+// against 108: their levels are wider than 16 CTAs. 128 unrelated matrices of up to 20 indices
+// take 195 us with this line at 8 or 9, 255 at 7.
+constexpr int kTreeSmallMax = 8;
+// Units (tasks of one CTA) that a launch aims at, per CTA that runs at a time, shared out by work:
+// a tree's work grows 2.26-fold with an index pair (n = 16 to 22). 512 patterns of up to 30
+// photons take 7.6 ms with 2, 7.06 with 4, 6.75 with 8, 6.63 with 16, and 10.0 with 2 shared
+// out evenly; the storage for the levels above the units grows with it.
+constexpr double kTreeUnits = 8;
+constexpr double kTreeGrowth = 2.26;
 constexpr int kTreeTop = 6;  // level from which a unit is worked off breadth first
 // Smallest scaled result that is kept. The tree's absolute error is about 2^-80 (against a
 // 113-bit evaluation), so 2^-28 leaves it at 2^-52 of the result. The subset sum it would be
@@ -480,7 +487,7 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
 
 // Small problems in one launch: a cluster of CTAs works a whole tree off breadth first, one
 // cluster barrier a level (a grid-wide step is a launch, 3 us; the levels of a small tree take
-// less). Its scratch holds every level.
+// less). Its scratch holds every level. Bound by the barriers and the latency of a level's loads.
 template <bool kOne>
 __global__ void __launch_bounds__(kRootThreads, 2)
 tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int first, int count,
@@ -569,11 +576,9 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
   auto pairs = [&](int q) { return std::max(4, Ns[T.order[q]] + (Ns[T.order[q]] & 1)) / 2; };
   // in launch order: large, small
   const int cluster_slots = 2 * dev.sm_count;
-  int alone = 0;
-  while (alone < count && pairs(count - 1 - alone) <= kTreeSmallMax) ++alone;
-  const int limit = alone * 8 <= cluster_slots ? kTreeSmallMax : kTreeSmallCrowd;
   T.nbig = 0;
-  while (T.nbig < count && pairs(T.nbig) > limit) ++T.nbig;
+  double work = 0;
+  while (T.nbig < count && pairs(T.nbig) > kTreeSmallMax) work += std::pow(kTreeGrowth, pairs(T.nbig++));
   const int nsmall = count - T.nbig;
   T.cluster = T.clusters = 0;
   T.small_bytes = 0;
@@ -601,8 +606,8 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
     P.root = root;
     if (q >= T.nbig) continue;
     P.m1 = n - 1;
-    const unsigned want = T.nbig == 1 ? 4 * slots : 2 * slots / (unsigned)T.nbig;
-    while (P.m1 > 2 && (unsigned)tree_width(P.m1, n) < want && n - P.m1 < (n > 24 ? 11 : 12)) --P.m1;
+    const double want = kTreeUnits * slots * std::pow(kTreeGrowth, n) / work;
+    while (P.m1 > 2 && tree_width(P.m1, n) < want && n - P.m1 < (n > 24 ? 11 : 12)) --P.m1;
     P.top = std::min(kTreeTop, P.m1);
     P.units = (unsigned)tree_width(P.m1, n);
     base += P.units;
