@@ -24,11 +24,20 @@ namespace gbsh {
 // ------------------------------------------------------------------ expansion
 // A0[r][c] = base[idx[r]][idx[c]] (r != c), v[r] = diag ? diag[idx[r]] : base[idx[r]][idx[r]].
 // Rows/columns >= N (odd padding) are zero with loop weight 1.
+// A gated evaluation's chunk counters are set here: zero if *gate is set, else past every chunk, so
+// that the subset kernels find nothing to claim. (A test of the flag in the subset kernels
+// themselves made every FP64 evaluation 3 % slower.)
 __global__ void expand_problem_kernel(const double2* __restrict__ base, int ld,
                                       const double2* __restrict__ diag,
                                       const int* __restrict__ idx, int N, int Ne,
-                                      double2* __restrict__ A0, double2* __restrict__ v) {
+                                      double2* __restrict__ A0, double2* __restrict__ v,
+                                      const unsigned* __restrict__ gate, unsigned* __restrict__ counters) {
+  chain_wait();
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  if (gate) {
+    if (tid < kMaxClasses) counters[tid] = *gate ? 0u : 0x80000000u;
+    if (*gate == 0) return;
+  }
   const int stride = gridDim.x * blockDim.x;
   for (int e = tid; e < Ne * Ne; e += stride) {
     int r = e / Ne, c = e - r * Ne;
@@ -148,6 +157,7 @@ __global__ void __launch_bounds__(kFinalizeThreads)
 lhaf_partials_kernel(const double* __restrict__ partials, unsigned nchunks, unsigned stride,
                      int nclass, double* __restrict__ block_out,
                      const unsigned* __restrict__ gate) {
+  chain_wait();
   if (gate && *gate == 0) return;
   __shared__ double sh[5][kFinalizeThreads];
   const unsigned per = (nchunks + gridDim.x - 1) / gridDim.x;
@@ -167,6 +177,7 @@ lhaf_partials_kernel(const double* __restrict__ partials, unsigned nchunks, unsi
 __global__ void __launch_bounds__(kFinalizeThreads)
 lhaf_finalize_kernel(const double* __restrict__ block_out, int nblocks, double* __restrict__ out,
                      double* __restrict__ value, const unsigned* __restrict__ gate) {
+  cudaGridDependencySynchronize();  // the last kernel of an evaluation: what follows is the caller's
   if (gate && *gate == 0) return;
   __shared__ double sh[5][kFinalizeThreads];
   DDAcc a;
@@ -184,13 +195,6 @@ lhaf_finalize_kernel(const double* __restrict__ block_out, int nblocks, double* 
       value[1] = out[1];
     }
   }
-}
-
-// Chunk counters of a gated evaluation: zero if *gate is set, else past every chunk, so that the
-// subset kernels find nothing to claim. (A test of the flag in the subset kernels themselves
-// made every FP64 evaluation 3 % slower.)
-__global__ void gate_counters_kernel(const unsigned* __restrict__ gate, unsigned* __restrict__ counters) {
-  counters[threadIdx.x] = *gate ? 0u : 0x80000000u;
 }
 
 // ================================================================== batched evaluation
@@ -492,15 +496,14 @@ static Problem problem_of(const LhafPlan& plan, void* ws) {
 
 static cudaError_t launch_expand(const LhafPlan& plan, const double2* base, int ld,
                                  const double2* diag, const int* idx, void* ws,
-                                 cudaStream_t stream) {
+                                 cudaStream_t stream, const unsigned* gate = nullptr) {
   char* b = static_cast<char*>(ws);
   const int elems = plan.Ne * plan.Ne;
   const int threads = 256;
   const int blocks = (elems + threads - 1) / threads;
-  expand_problem_kernel<<<blocks, threads, 0, stream>>>(
-      base, ld, diag, idx, plan.N, plan.Ne, reinterpret_cast<double2*>(b + plan.off_A0),
-      reinterpret_cast<double2*>(b + plan.off_v));
-  return cudaGetLastError();
+  return launch_chained(expand_problem_kernel, blocks, threads, stream, gate != nullptr, base, ld, diag, idx, plan.N, plan.Ne,
+                        reinterpret_cast<double2*>(b + plan.off_A0), reinterpret_cast<double2*>(b + plan.off_v),
+                        gate, reinterpret_cast<unsigned*>(b + plan.off_counters));
 }
 
 // Side streams on which the popcount classes after the first run, so that the tail of one
@@ -534,17 +537,12 @@ static cudaError_t side_streams(cudaStream_t** out) {
 template <bool kVisit>
 static cudaError_t launch_classes(const LhafPlan& plan, void* ws, unsigned* visits,
                                   cudaStream_t stream, uint64_t i_base, uint64_t i_end,
-                                  unsigned nchunks, const unsigned* gate = nullptr) {
+                                  unsigned nchunks, bool gated = false) {
   char* b = static_cast<char*>(ws);
   unsigned* counters = reinterpret_cast<unsigned*>(b + plan.off_counters);
   double* partials = reinterpret_cast<double*>(b + plan.off_partials);
   cudaError_t e = cudaSuccess;
-  if (gate) {
-    gate_counters_kernel<<<1, kMaxClasses, 0, stream>>>(gate, counters);
-    e = cudaGetLastError();
-  } else {
-    e = cudaMemsetAsync(counters, 0, sizeof(unsigned) * kMaxClasses, stream);
-  }
+  if (!gated) e = cudaMemsetAsync(counters, 0, sizeof(unsigned) * kMaxClasses, stream);
   if (e != cudaSuccess) return e;
   const Problem P = problem_of(plan, ws);
   cudaStream_t* side = nullptr;
@@ -589,21 +587,21 @@ cudaError_t launch_range(const LhafPlan& plan, const double2* base, int ld,
                          const double2* diag, const int* idx, void* ws,
                          cudaStream_t stream, uint64_t i_begin, uint64_t i_end,
                          const unsigned* gate, double* value) {
-  cudaError_t e = launch_expand(plan, base, ld, diag, idx, ws, stream);
+  cudaError_t e = launch_expand(plan, base, ld, diag, idx, ws, stream, gate);
   if (e != cudaSuccess) return e;
   const uint64_t span = i_end > i_begin ? i_end - i_begin : 0;
   const unsigned nchunks = (unsigned)((span + plan.chunk_size - 1) / plan.chunk_size);
-  e = launch_classes<false>(plan, ws, nullptr, stream, i_begin, i_end, nchunks, gate);
+  e = launch_classes<false>(plan, ws, nullptr, stream, i_begin, i_end, nchunks, gate != nullptr);
   if (e != cudaSuccess) return e;
   char* b = static_cast<char*>(ws);
   double* blocks = reinterpret_cast<double*>(b + plan.off_blocks);
-  lhaf_partials_kernel<<<kReduceBlocks, kFinalizeThreads, 0, stream>>>(
-      reinterpret_cast<const double*>(b + plan.off_partials), nchunks, plan.nchunks, plan.nclass,
-      blocks, gate);
-  lhaf_finalize_kernel<<<1, kFinalizeThreads, 0, stream>>>(blocks, kReduceBlocks,
-                                                           reinterpret_cast<double*>(b + plan.off_out), value,
-                                                           gate);
-  return cudaGetLastError();
+  // several classes end on other streams
+  e = launch_chained(lhaf_partials_kernel, kReduceBlocks, kFinalizeThreads, stream, plan.nclass == 1,
+                     reinterpret_cast<const double*>(b + plan.off_partials), nchunks, plan.nchunks,
+                     plan.nclass, blocks, gate);
+  if (e != cudaSuccess) return e;
+  return launch_chained(lhaf_finalize_kernel, 1, kFinalizeThreads, stream, true, blocks, kReduceBlocks,
+                        reinterpret_cast<double*>(b + plan.off_out), value, gate);
 }
 
 cudaError_t launch_lhaf(const LhafPlan& plan, const double2* base, int ld, const double2* diag,

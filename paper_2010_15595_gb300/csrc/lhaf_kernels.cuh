@@ -108,4 +108,34 @@ cudaError_t launch_batch(const BatchInput* d_in, const BatchProblem* d_prob, int
                          int warps_small, unsigned* d_counter, double* d_partials, double* d_out,
                          cudaStream_t stream, cudaStream_t side_stream = nullptr);
 
+// Launches `k`; if `chained`, so that its CTAs may start while the launch before it on the stream
+// ends: the kernel itself waits for that one's results (chain_wait). Only directly after a kernel
+// of this library that was launched the plain way or waits in the same manner.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*k)(P...), dim3 grid, int threads, cudaStream_t st,
+                           bool chained, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
+#ifdef __CUDACC__
+// Start of a kernel of a chain: lets the next launch of the stream start its CTAs (they wait here in
+// turn), and waits until the launch before has ended and its writes can be seen. Each kernel of
+// the chain waits before it touches memory, so all earlier ones have ended too. A level of the
+// tree is a launch of 3 to 6 us; started this way, N = 16 takes 42 us instead of 52, N = 20 61
+// instead of 84, N = 32 339 instead of 361.
+__device__ __forceinline__ void chain_wait() {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+}
+#endif
+
 }  // namespace gbsh

@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kRootThreads)
 tree_root_kernel(const TreeProblem* __restrict__ table, TreeProblem one, TreeState* __restrict__ state,
                  unsigned* __restrict__ counter, char* __restrict__ levels) {
   __shared__ RootShared sh;
+  cudaTriggerProgrammaticLaunchCompletion();  // launched the plain way: nothing to wait for
   const TreeProblem P = kOne ? one : table[blockIdx.x];
   if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
   tree_root<kRootThreads>(P, tree_level(levels + P.root, P.n, P.n, 1), state + blockIdx.x, sh);
@@ -370,6 +371,7 @@ tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ 
                  TreeState* __restrict__ state, char* __restrict__ levels) {
   __shared__ TreePhase many;
   __shared__ int slots[kSlotInts][kTreeThreads];
+  chain_wait();
   if (!kOne) {
     if (table[blockIdx.y].n - step <= table[blockIdx.y].m1) return;  // fewer steps than another's
     if (threadIdx.x == 0)
@@ -433,6 +435,7 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
   __shared__ int s_prob;
   const int tid = threadIdx.x;
   char* ws = scratch + (size_t)blockIdx.x * cta_bytes;
+  chain_wait();
   for (;;) {
     if (tid == 0) {
       const unsigned u = atomicAdd(counter, 1u);
@@ -659,22 +662,17 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
       tree_root_kernel<true><<<1, kRootThreads, 0, st>>>(table, p0, state, counter, levels);
     else
       tree_root_kernel<false><<<plan.nbig, kRootThreads, 0, st>>>(table, p0, state, counter, levels);
-    for (int i = 0; i < (int)plan.steps.size(); ++i) {
+    e = cudaGetLastError();
+    for (int i = 0; i < (int)plan.steps.size() && e == cudaSuccess; ++i) {
       const dim3 grid((plan.steps[i].tasks + kTreeThreads - 1) / kTreeThreads, plan.steps[i].problems);
       const TreePhase s = tree_whole_phase(levels + p0.root, p0.n, i);
-      if (one)
-        tree_step_kernel<true><<<grid, kTreeThreads, 0, st>>>(table, s, i, plan.fine, state, levels);
-      else
-        tree_step_kernel<false><<<grid, kTreeThreads, 0, st>>>(table, s, i, plan.fine, state, levels);
+      e = launch_chained(one ? tree_step_kernel<true> : tree_step_kernel<false>, grid, kTreeThreads, st, true, table, s, i,
+                         plan.fine, state, levels);
     }
-    if (one)
-      tree_kernel<true><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, 1, plan.total_units, state, counter,
-                                                              levels, scratch, plan.cta_bytes, out, flags);
-    else
-      tree_kernel<false><<<plan.blocks, kTreeThreads, 0, st>>>(table, p0, plan.nbig, plan.total_units, state,
-                                                               counter, levels, scratch, plan.cta_bytes, out,
-                                                               flags);
-    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = launch_chained(one ? tree_kernel<true> : tree_kernel<false>, dim3(plan.blocks), kTreeThreads, st, true, table,
+                         p0, plan.nbig, plan.total_units, state, counter, levels, scratch, plan.cta_bytes, out,
+                         flags);
   }
   if (e == cudaSuccess && plan.nbig < count) {
     const auto k = one ? tree_small_kernel<true> : tree_small_kernel<false>;
