@@ -644,17 +644,16 @@ cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStrea
                          sizeof(TreeProblem) * plan->prob.size(), cudaMemcpyHostToDevice, st);
 }
 
-cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* value) {
+cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* out, bool flags) {
   const int count = (int)plan.prob.size();
   if (count == 0) return cudaSuccess;
   char* b = static_cast<char*>(ws);
-  const bool one = count == 1, flags = value == nullptr;
+  const bool one = count == 1;
   const TreeProblem* table = one ? nullptr : reinterpret_cast<const TreeProblem*>(b + plan.off_prob);
   TreeState* state = reinterpret_cast<TreeState*>(b + plan.off_state);
   unsigned* counter = reinterpret_cast<unsigned*>(b + plan.off_counter);
   char* levels = b + plan.off_root;
   char* scratch = b + plan.off_cta;
-  double* out = value ? value : reinterpret_cast<double*>(b + plan.off_out);
   const TreeProblem& p0 = plan.prob[0];
   cudaError_t e = cudaSuccess;
   if (plan.nbig > 0) {
@@ -696,15 +695,18 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
   return e;
 }
 
-cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st, double* out3,
-                     std::vector<int>* again) {
+cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host, cudaStream_t st,
+                     double* out3, std::vector<int>* again) {
   const size_t count = plan->prob.size();
-  std::vector<double> res(3 * count);
+  // The kernels write the results straight to page-locked memory: with a copy to pageable memory
+  // instead (and the matrix of gbsh_lhaf copied from there), a call takes 75 us at N = 16, not 61.
+  std::vector<double> pageable(host ? 0 : 3 * count);
+  double* res = host ? static_cast<double*>(host) : pageable.data();
+  double* out = host ? res : reinterpret_cast<double*>(static_cast<char*>(ws) + plan->off_out);
   cudaError_t e = tree_stage(plan, in, ws, st);
-  if (e == cudaSuccess) e = tree_launch(*plan, ws, st);
-  if (e == cudaSuccess && count > 0)
-    e = cudaMemcpyAsync(res.data(), static_cast<char*>(ws) + plan->off_out, sizeof(double) * res.size(),
-                        cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = tree_launch(*plan, ws, st, out, true);
+  if (e == cudaSuccess && !host && count > 0)
+    e = cudaMemcpyAsync(res, out, sizeof(double) * 3 * count, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return e;
   for (size_t q = 0; q < count; ++q) {

@@ -53,18 +53,19 @@ struct TreePlan {
 cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan);
 
 // Evaluates the problems of `plan` (in[i]: input of the caller's problem i) in `ws` on `st`.
-// Result of launch-order problem q: three doubles at off_out + 24 q: re, im, and 1 where the
-// problem has to be evaluated by the subset sum instead (0 otherwise). `value` (one-problem
-// launches): device pointer that receives re, im instead; the flag is then at tree_flag().
-cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* value = nullptr);
+// Result of launch-order problem q, if `flags`: three doubles at out + 3 q: re, im, and 1 where
+// the problem has to be evaluated by the subset sum instead (0 otherwise). Without (one-problem
+// launches): re, im, and the flag at tree_flag().
+cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* out, bool flags);
 
 // Fills in the inputs and, for more than one problem, uploads the table.
 cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st);
 
 // Stages and launches `plan`, waits, and copies the results to out3[3 i ..] of the caller's
 // problem i (re, im, 0); problems to be evaluated by the subset sum are added to `again`.
-cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st, double* out3,
-                     std::vector<int>* again);
+// `host`: page-locked memory of at least 24 bytes a problem that the call may use, or null.
+cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host, cudaStream_t st,
+                     double* out3, std::vector<int>* again);
 
 // Device address of a one-problem launch's fallback flag (nonzero: evaluate by the subset sum).
 const unsigned* tree_flag(const TreePlan& plan, void* ws);

@@ -218,6 +218,7 @@ struct gbsh_sampler {
   size_t idx_cap = 0;
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  char* host = nullptr;  // kHostBytes of page-locked memory for a tick's results, or null
   double* dpart = nullptr;  // range partials of one tick (5 doubles each)
   size_t part_cap = 0;
   std::vector<int> free_slots;
@@ -232,6 +233,8 @@ struct gbsh_sampler {
 };
 
 namespace {
+
+constexpr size_t kHostBytes = 64 << 10;
 
 int from_cuda(cudaError_t e) {
   return e == cudaSuccess ? GBSH_OK : (e == cudaErrorMemoryAllocation ? GBSH_ENOMEM : GBSH_ECUDA);
@@ -411,7 +414,8 @@ int gbsh_sampler::tick(std::vector<Chain>& active) {
       for (size_t q = 0; q < m; ++q) some[q] = in[sel[f + q]];
       std::vector<double> o(3 * m);
       std::vector<int> again;
-      e = gbsh::tree_run(&T, some.data(), ws, st, o.data(), &again);
+      e = gbsh::tree_run(&T, some.data(), ws, sizeof(double) * o.size() <= kHostBytes ? host : nullptr, st,
+                         o.data(), &again);
       if (e != cudaSuccess) return from_cuda(e);
       for (size_t q = 0; q < m; ++q)
         for (int j = 0; j < 3; ++j) out3[3 * (size_t)sel[f + q] + j] = o[3 * q + j];
@@ -786,6 +790,10 @@ int gbsh_sampler_create(const gbsh_sampler_cfg* cfg, gbsh_sampler** out) {
   if ((e = cudaMalloc(&h->dk, sizeof(int) * slots)) != cudaSuccess) return fail(e);
   if ((e = cudaMemcpy(h->dB, h->B.data(), sizeof(double2) * M * M, cudaMemcpyHostToDevice)) != cudaSuccess)
     return fail(e);
+  if (cudaMallocHost(reinterpret_cast<void**>(&h->host), kHostBytes) != cudaSuccess) {
+    cudaGetLastError();
+    h->host = nullptr;
+  }
   cudaSetDevice(prev);
   gbsh_sampler* raw = h.release();
   raw->worker = std::thread([raw] { raw->run(); });
@@ -897,6 +905,7 @@ int gbsh_sampler_destroy(gbsh_sampler* h) {
   cudaFree(h->didx);
   cudaFree(h->dpart);
   cudaFree(h->ws);
+  cudaFreeHost(h->host);
   if (h->st) cudaStreamDestroy(h->st);
   cudaSetDevice(prev);
   delete h;
