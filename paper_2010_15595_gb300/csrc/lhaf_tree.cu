@@ -27,8 +27,13 @@ namespace gbsh {
 
 namespace {
 
+// CTAs of tree_step_kernel and tree_kernel. 5 of 128 threads leave 96 registers a thread, which
+// hold fx_conv2's operands a step ahead: N = 32 318 us and 512 patterns of up to 30 photons
+// 6.38 ms, against 338 us and 6.71 ms with 6 (80 registers, nothing loaded ahead), 324 us and
+// 6.77 ms with 4 (N = 44: 22.1, 22.0, 23.0 ms). Other widths (64 to 256 threads) were 4 to 28 %
+// slower at N = 40.
 constexpr int kTreeThreads = 128;
-constexpr int kTreeCtasPerSm = 6;
+constexpr int kTreeCtasPerSm = 5;
 // Largest n of a small problem (tree_small_kernel). Alone, n = 8 takes 53 us that way against 72
 // by launches; n = 9 and 10 the same either way, n = 11 takes 104 against 91 and n = 12 162
 // against 108: their levels are wider than 16 CTAs. 128 unrelated matrices of up to 20 indices
@@ -40,7 +45,9 @@ constexpr int kTreeSmallMax = 8;
 // out evenly; the storage for the levels above the units grows with it.
 constexpr double kTreeUnits = 8;
 constexpr double kTreeGrowth = 2.26;
-constexpr int kTreeTop = 6;  // level from which a unit is worked off breadth first
+// Level from which a unit is worked off breadth first: 5 takes 5.31 ms at N = 40 (levels too narrow
+// for a CTA), 7 takes 23.6 ms at N = 44 (its storage leaves the L2), 6 takes 4.7 and 22.0.
+constexpr int kTreeTop = 6;
 // Smallest scaled result that is kept. The tree's absolute error is about 2^-80 (against a
 // 113-bit evaluation), so 2^-28 leaves it at 2^-52 of the result. The subset sum it would be
 // handed back to is itself 2^-47 off at N = 32, 2^-42 at N = 40 and 2^-31 at N = 56, so the line
@@ -270,7 +277,9 @@ __device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState
   if (tid == 0) S->bad = any ? 1 : 0;
 }
 
-// kOne: one problem, passed as a kernel argument; otherwise a table in device memory.
+// Scales a problem and makes its level n. One CTA a problem: 8 to 13 us of dependent steps (norms,
+// scale, conversion), hidden in a batch. kOne: one problem, passed as a kernel argument;
+// otherwise a table in device memory.
 template <bool kOne>
 __global__ void __launch_bounds__(kRootThreads)
 tree_root_kernel(const TreeProblem* __restrict__ table, TreeProblem one, TreeState* __restrict__ state,
@@ -363,8 +372,10 @@ struct JobSlot {
   __device__ __forceinline__ int get(int k) const { return m[k][threadIdx.x]; }
 };
 
-// kOne: the phase of the one problem is set up on the host. Phases of at most `fine` pieces run in
-// pieces.
+// One breadth-first level of the large problems, the whole GPU on it: 3 to 17 us, the latency of a
+// launch and of its loads for the narrow levels, the products for the wide ones. kOne: the phase
+// of the one problem is set up on the host. Phases of at most `fine` pieces, a quarter of a
+// coefficient a thread, run that way: a narrow level is as long as one thread's work.
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ TreePhase one, int step, int fine,
@@ -422,6 +433,12 @@ struct LimbSums {
   }
 };
 
+// The units of all large problems, claimed from a counter by one resident wave of CTAs: nearly all
+// of a large evaluation. A unit's levels live in the CTA's own scratch (walked depth first, two
+// nodes a level, so that the scratch of all CTAs stays in the L2) and its tasks are independent
+// within a phase. Bound by the convolutions' multiply-adds (70 %, see fx_conv2) and the latency of
+// their loads (43 % hit L1, and a warp waits for one during 27 % of its time). N = 40: 4.65 ms, 0.22e12 complex
+// multiply-adds/s (184 ms for the subset sum); N = 44: 21.6 ms (919).
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, unsigned total_units,
@@ -490,7 +507,8 @@ tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, u
 
 // Small problems in one launch: a cluster of CTAs works a whole tree off breadth first, one
 // cluster barrier a level (a grid-wide step is a launch, 3 us; the levels of a small tree take
-// less). Its scratch holds every level. Bound by the barriers and the latency of a level's loads.
+// less). Its scratch holds every level. Bound by the barriers and the latency of a level's loads:
+// N = 16 takes 31 us (42 with the gated launches behind it; 135 by the subset sum).
 template <bool kOne>
 __global__ void __launch_bounds__(kRootThreads, 2)
 tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int first, int count,

@@ -20,20 +20,21 @@
 //
 // Work: 2^{n-3} leaves with about 62 products of truncated polynomials each, ~8 n^2 2^n / 15
 // complex multiply-adds in all, against ~n^3 2^n for building every subset term from scratch
-// (N = 40: 1.1e9 against 1.1e10), and the signed mean cancels by 10^2..10^4 where the signed
+// (N = 40: 1.0e9 against 1.1e10, 4.7 ms against 184), and the signed mean cancels by 10^2..10^4 where the signed
 // subset sum cancels by 10^7..10^12.
 //
 // Arithmetic. Products of polynomials are sums of products with no division, so they run in
 // fixed point: a real number is an integer times 2^-81, held as three limbs with signs,
 // h 2^54 + m 2^27 + l, |m|, |l| <= 2^26, |h| < 2^29. The limb products of a whole convolution
 // add up in 64 bits, so it accumulates exactly and is normalised once. Six limb products per real
-// product (the three below 2^-81 are dropped) make 24 32x32+64-bit integer multiply-adds per
-// complex one: 0.35e12 complex multiply-adds/s with operands from L1, against 0.17e12/s at best
-// for triple-float (216 FP32 instructions) and 0.15e12/s for FP64. (The integer multiply-add
-// issues every 2 cycles when it repeats its operands, 18.7e12/s, and every 4.4 in this code; its
-// operand fetch is the limit of the whole evaluation.) Fixed point needs a scale: the matrix is
-// scaled by one factor such that its root-mean-fourth singular value is about one, which keeps
-// the coefficients of every matrix tried between 2^-10 and 2.5 (the format holds |x| < 4).
+// product (the three below 2^-81 are dropped) and three real products per complex one (Gauss) make
+// 18 32x32+64-bit integer multiply-adds per complex one: 0.45e12 complex multiply-adds/s with
+// operands from L1, against 0.17e12/s at best for triple-float (216 FP32 instructions) and
+// 0.15e12/s for FP64. (The integer multiply-add issues every 2 cycles when it repeats its
+// operands, 18.7e12/s, and every 4.4 in this code: its operand fetch is the limit.) Fixed point
+// needs a scale: the matrix is scaled by one factor such that its root-mean-fourth singular value
+// is about one, which keeps the coefficients of every matrix tried between 2^-10 and 2.5 (the
+// format holds |x| < 4).
 // Overflow anywhere, or a result so small that the 2^-81 resolution could show, sets a flag and
 // the caller evaluates the problem by the subset sum instead.
 //
@@ -98,8 +99,8 @@ struct FxSum {
 };
 // Such sums while they grow: p = sum of re re, q = sum of im im, t = sum of (re + im) (re + im),
 // from which re = p - q and im = t - p - q (Gauss): 18 multiply-adds a complex product instead of
-// 24. The products alone run at 450 against 350 G complex multiply-adds/s; in tree_kernel N = 40
-// takes 4.72 ms instead of 5.00. t may wrap in 64 bits; the differences fit. The sums start at
+// 24. The products alone run at 450 against 350 G complex multiply-adds/s; with it N = 40 took
+// 4.72 ms instead of 5.00. t may wrap in 64 bits; the differences fit. The sums start at
 // half a unit of the next limb, which turns the cuts in fx_norm into roundings to the nearest.
 struct FxAcc {
   long long p2, p1, p0, q2, q1, q0, t2, t1, t0;
@@ -175,21 +176,24 @@ GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, unsigned& bad) {
 // acc0, acc1 += coefficients t0, t0 + 1 of the polynomial product a * b, coefficient u at a + u sa
 // and b + u sb; t0 = -1 leaves acc0 alone. t0 + 1 must not exceed the last coefficient of either
 // factor. Two coefficients a task: each step loads one new element of each factor for two
-// multiply-adds (b in a sliding window of two). Four would halve the loads, but with the
-// accumulators of four (48 registers) the code spilled and outgrew the instruction cache
-// (N = 40: 9.0 ms against 5.7 ms).
+// multiply-adds (b in a sliding window of two, a one step ahead of its use). Four would halve the
+// loads, but with the accumulators of four the code spilled and outgrew the instruction cache
+// (N = 40: 9.0 ms against 5.7 ms). Bound by how fast the register file feeds the 64-bit
+// multiply-adds: one a warp and 4.4 cycles, not the 2 of a chain on fixed registers, whatever the
+// order of operands or the pairing of registers.
 GBSH_HD void fx_conv2(FxAcc& acc0, FxAcc& acc1, const char* a, int sa, const char* b, int sb, int t0) {
   b += (ptrdiff_t)(t0 + 1) * sb;
-  Fxc w1 = fx_load(b), w0{};
+  Fxc w1 = fx_load(b), x = fx_load(a), w0{};
   int u = t0 + 1;  // steps before the last one
   if (u > 0) {
     b -= sb;
     w0 = fx_load(b);
     if (u & 1) {
-      const Fxc x = fx_load(a);
       a += sa;
+      const Fxc y = fx_load(a);
       fx_mac(acc0, x, w0);
       fx_mac(acc1, x, w1);
+      x = y;
       w1 = w0;
       if (u > 1) {
         b -= sb;
@@ -200,23 +204,23 @@ GBSH_HD void fx_conv2(FxAcc& acc0, FxAcc& acc1, const char* a, int sa, const cha
 #pragma unroll 1
 #endif
     for (u >>= 1; u > 0; --u) {
-      Fxc x = fx_load(a);
       a += sa;
-      fx_mac(acc0, x, w0);
+      const Fxc y = fx_load(a);
       fx_mac(acc1, x, w1);
       b -= sb;
       w1 = fx_load(b);
-      x = fx_load(a);
+      fx_mac(acc0, x, w0);
       a += sa;
-      fx_mac(acc0, x, w1);
-      fx_mac(acc1, x, w0);
+      x = fx_load(a);
+      fx_mac(acc1, y, w0);
       if (u > 1) {
         b -= sb;
         w0 = fx_load(b);
       }
+      fx_mac(acc0, y, w1);
     }
   }
-  fx_mac(acc1, fx_load(a), w1);
+  fx_mac(acc1, x, w1);
 }
 
 // ------------------------------------------------------------------ levels of the tree
@@ -510,7 +514,7 @@ GBSH_HD int tree_pieces(const TreePhase& s) { return (s.n - s.M + 1) * s.items *
 
 // The parts of a job that a task does not need during its products, kept outside the registers
 // (on the GPU in shared memory, a column per thread): two FxAcc and three operands with their
-// sums take 63 of the 80 registers that 768 threads an SM leave.
+// sums take 63 of the 96 registers that 640 threads an SM leave.
 constexpr int kSlotInts = 11;
 template <class Slot>
 GBSH_HD void tree_put(const Slot& m, const TreeJob& J) {
