@@ -580,6 +580,8 @@ tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int fi
   }
 }
 
+constexpr int kMaxGridY = 65535;
+
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -681,10 +683,13 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
       tree_root_kernel<false><<<plan.nbig, kRootThreads, 0, st>>>(table, p0, state, counter, levels);
     e = cudaGetLastError();
     for (int i = 0; i < (int)plan.steps.size() && e == cudaSuccess; ++i) {
-      const dim3 grid((plan.steps[i].tasks + kTreeThreads - 1) / kTreeThreads, plan.steps[i].problems);
       const TreePhase s = tree_whole_phase(levels + p0.root, p0.n, i);
-      e = launch_chained(one ? tree_step_kernel<true> : tree_step_kernel<false>, grid, kTreeThreads, st, true, table, s, i,
-                         plan.fine, state, levels);
+      const unsigned x = (unsigned)(plan.steps[i].tasks + kTreeThreads - 1) / kTreeThreads;
+      for (int f = 0; f < plan.steps[i].problems && e == cudaSuccess; f += kMaxGridY) {
+        const dim3 grid(x, (unsigned)std::min(plan.steps[i].problems - f, kMaxGridY));
+        e = launch_chained(one ? tree_step_kernel<true> : tree_step_kernel<false>, grid, kTreeThreads, st, true,
+                           one ? table : table + f, s, i, plan.fine, state + f, levels);
+      }
     }
     if (e == cudaSuccess)
       e = launch_chained(one ? tree_kernel<true> : tree_kernel<false>, dim3(plan.blocks), kTreeThreads, st, true, table,

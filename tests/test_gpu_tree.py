@@ -26,8 +26,8 @@ def _async(gbsh, A, prec, nbytes=None):
     return complex(out.item())
 
 
-# 1..6: padding to four vertices, no signed pair, one signed pair; 8, 10, 12, 16, 18: cluster
-# sizes of the small kernel; 24, 25, 26: its last size and the first ones of the other kernels
+# 1..6: padding to four vertices, no signed pair, one signed pair; 8, 10, 12, 16: cluster sizes of
+# the small kernel, 16 its last size; 18 on: the other kernels; 24, 25: the last FP64 size and after
 @pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 13, 16, 18, 19, 23, 24, 25, 26])
 def test_sizes_and_entry_points(gbsh, N):
     rng = np.random.default_rng(700 + N)
@@ -109,6 +109,13 @@ def test_workspace_of_the_subset_sum_is_still_taken(gbsh):
         v = _async(gbsh, A, prec, nbytes=small)
         subset, _ = gbsh.lhaf(A, precision=prec, return_error=True)
         assert v == subset
+
+
+def test_more_large_problems_than_a_grid_has_rows(gbsh):
+    """A level's launch has a row of CTAs per problem, at most 65535."""
+    A = W.single_lhaf_mid(18)[:17, :17]
+    v = gbsh.lhaf_batch([A] * 65540, precision=gbsh.PREC_TF)
+    assert np.all(v == gbsh.lhaf(A, precision=gbsh.PREC_TF))
 
 
 def test_graph_capture(gbsh):
