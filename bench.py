@@ -5,9 +5,11 @@ Workload (one step): the loop hafnian of one N=40 complex symmetric matrix per G
 M=40 modes, Haar-random interferometer, squeezing r_i ~ U[0.4, 0.9], B = U diag(tanh r) U^T
 with the diagonal replaced by gamma_i ~ CN(0, 0.2^2) -- i.e. the 2^20 pair-subset terms of
 the subset formula. Metric: subset-terms per second (whole job). The headline path is the
-accurate one (triple-float per subset, which meets the stated relative tolerance), with the
-FP32-issue roofline fraction of its subset kernel; the FP64 path is timed beside it with its
-FP64 roofline fraction, and each path's error against the oracle's reference is reported.
+accurate one as a user calls it (GBSH_PREC_TF, which meets the stated relative tolerance): the
+elimination tree, which evaluates the sum of those terms without visiting them one by one, with
+the integer multiply-add roofline fraction of its work. Beside it: the same precision with the
+error estimate (sum |p_Z|), for which the subset sum visits every term, with its FP32-issue
+fraction; the FP64 path with its FP64 fraction; and each path's error against the oracle.
 Each rank evaluates its own seeded matrix (weak scaling, no data-path collective). Shorter
 measurements at N=50 (2^25 subsets) are reported under "n50".
 
@@ -136,6 +138,7 @@ class ClockSampler:
 # C-ABI wrappers do not change what one evaluation moves through DRAM).
 KERNEL_SOURCES = ("lhaf_core.cuh", "lhaf_kernels.cu", "lhaf_kernels.cuh", "lhaf_types.cuh",
                   "lhaf_tf.cuh", "tuned_gb300.inc")
+TREE_SOURCES = ("lhaf_tree.cuh", "lhaf_tree.cu", "lhaf_tree.h", "lhaf_types.cuh")
 
 
 def tuning_block(N: int) -> dict:
@@ -149,30 +152,50 @@ def tuning_block(N: int) -> dict:
             "batch_fp64_n15": dict(zip(("warps_small", "warps_large"), lib.get_batch_tuning(lib.PREC_FP64, 15)))}
 
 
-def kernel_source_hash() -> str:
+def kernel_source_hash(files=KERNEL_SOURCES) -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2010_15595_gb300", "csrc")
-    for f in KERNEL_SOURCES:
+    for f in files:
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
 def recorded_traffic(N: int, path: str, whole: bool = False):
-    """DRAM bytes per evaluation on `path` ("tf" or "fp64") from the committed ncu summary, if
-    it was taken on the current kernel sources (else None): the subset kernel's class launches
-    (the dominant kernel), or with whole=True every launch of the evaluation (expansion,
-    class launches, the two finalize levels)."""
-    p = os.path.join(ROOT, "profiles", "lhaf_subsets_dram_traffic.json")
+    """DRAM bytes per evaluation on `path` ("tree", or "tf" and "fp64" of the subset sum) from the
+    committed ncu summary, if it was taken on the current kernel sources (else None): the
+    dominant kernel (the tree kernel; the subset kernel's class launches), or with whole=True
+    every launch of the evaluation."""
+    p = os.path.join(ROOT, "profiles", "lhaf_%s_dram_traffic.json" % ("tree" if path == "tree" else "subsets"))
     try:
         with open(p) as f:
             rec = json.load(f)
     except (OSError, ValueError):
         return None
-    if rec.get("kernel_source_hash") != kernel_source_hash():
+    if rec.get("kernel_source_hash") != kernel_source_hash(TREE_SOURCES if path == "tree" else KERNEL_SOURCES):
         return None
+    if path == "tree":
+        return rec["bytes_per_evaluation" if whole else "tree_kernel_bytes_per_evaluation"].get(str(N))
     key = "bytes_per_evaluation" if whole else "subset_kernel_bytes_per_evaluation"
     return rec.get(key, {}).get(path, {}).get(str(N))
+
+
+def kernel_launches(fn) -> int:
+    """Kernels that one call of `fn` launches, counted by the profiler. Only after everything
+    timed: launches stay slower in a process that has profiled."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):  # the first activities of a process may not be recorded
+        fn()
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            fn()
+            torch.cuda.synchronize()
+        count = sum(e.device_type == torch.autograd.DeviceType.CUDA and not e.name.startswith("Mem")
+                    for e in p.events())
+        if count:
+            return count
+    return 0
 
 
 def recorded_probes() -> dict:
@@ -259,12 +282,13 @@ def run_ours(args, rank, world, local_rank):
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     ref40 = golden_reference("lhaf_n40") if (rank == 0 and N == 40) else None
 
-    def timed_path(prec, steps, warmup):
+    def timed_path(prec, steps, warmup, abs_sum):
         """Times `steps` evaluations of the step matrix in `prec` (CUDA events on the
-        launching stream, L2 flushed between steps outside the events)."""
+        launching stream, L2 flushed between steps outside the events). abs_sum: with sum |p_Z|
+        (the error estimate), which only the subset sum gives."""
         ws = torch.empty(lib.workspace_size(N, prec), dtype=torch.uint8, device=dev)
         out = torch.empty(1, dtype=torch.complex128, device=dev)
-        asum = torch.empty(1, dtype=torch.float64, device=dev)
+        asum = torch.empty(1, dtype=torch.float64, device=dev) if abs_sum else None
 
         def step():
             lib.lhaf_async(dA, out, ws, d_abs_sum=asum, stream=stream, precision=prec)
@@ -290,21 +314,43 @@ def run_ours(args, rank, world, local_rank):
         total_s = max_over_ranks(sum(step_ms) / 1e3, dev)
         v = complex(out.item())
         return {"total_s": total_s, "mean_s": statistics.mean(step_ms) / 1e3, "wall": wall,
-                "clocks": clocks.summary(), "lhaf": v, "abs_sum": float(asum.item())}
+                "clocks": clocks.summary(), "lhaf": v, "step": step,
+                "abs_sum": float(asum.item()) if abs_sum else None}
 
     subsets = workmodel.subset_count(N)
-    tf_run = timed_path(TF, args.steps, args.warmup)
-    fp_run = timed_path(F64, args.steps, args.warmup)
+    tf_run = timed_path(TF, args.steps, args.warmup, False)
+    sum_steps = min(args.steps, 5)
+    sum_run = timed_path(TF, sum_steps, args.warmup, True)
+    fp_run = timed_path(F64, args.steps, args.warmup, True)
     ms_per_step = tf_run["total_s"] * 1e3 / args.steps
     value = subsets * world * args.steps / tf_run["total_s"]
+    imads = workmodel.tree_macs(N) * workmodel.TREE_IMAD
+    imad_ach = imads / tf_run["mean_s"] / 1e12
+    imad_peak = workmodel.IMAD_PEAK_DERIVED_T
     tf_instr = workmodel.lhaf_tf_instr(N)
-    tf_ach = tf_instr / tf_run["mean_s"] / 1e12
+    tf_ach = tf_instr / sum_run["mean_s"] / 1e12
     tf_peak = workmodel.FP32_INSTR_PEAK_DERIVED_T
     flops = workmodel.lhaf_flops(N)
     sflops = workmodel.householder_flops(N)
     fp_ach = flops / fp_run["mean_s"] / 1e12
     fp_peak = workmodel.FP64_PEAK_DERIVED_TFLOPS
     probes = recorded_probes()
+    subset_sum = {"value": subsets * world * sum_steps / sum_run["total_s"], "unit": UNIT,
+                  "ms_per_step": sum_run["total_s"] * 1e3 / sum_steps, "steps": sum_steps,
+                  "path": "triple-float per subset (three FP32 words, ~72-bit significand), every "
+                          "subset visited, compensated FP64 cross-subset sum; with sum |p_Z|",
+                  "plan": lib.plan(N, TF),
+                  "roofline": {"bound": "alu", "achieved": tf_ach, "peak": tf_peak,
+                               "unit": "T FP32 instr/s", "frac": tf_ach / tf_peak,
+                               "traffic": recorded_traffic(N, "tf"),
+                               "traffic_whole_evaluation": recorded_traffic(N, "tf", whole=True),
+                               "peak_source": "derived: 152 SM x 128 FP32 lanes/clk x 2.07 GHz",
+                               "measured_ffma_probe_t_instr": probes.get("ffma_t_instr"),
+                               "kernel": "lhaf_subsets_kernel<tfc> (+expand, finalize in the step time)",
+                               "work_per_launch": tf_instr,
+                               "work_convention": "FP32 arithmetic instructions of the triple-float "
+                                                  "algorithm (216 per complex multiply-add)"},
+                  "clocks": sum_run["clocks"]}
     fp64 = {"value": subsets * world * args.steps / fp_run["total_s"], "unit": UNIT,
             "ms_per_step": fp_run["total_s"] * 1e3 / args.steps,
             "roofline": {"bound": "alu", "achieved": fp_ach, "peak": fp_peak, "unit": "TFLOP/s",
@@ -373,11 +419,13 @@ def run_ours(args, rank, world, local_rank):
         sec = e0.elapsed_time(e1) / 1e3
         v = complex(oL.item())
         res = {"seconds": sec, "value": workmodel.subset_count(N_) / sec, "unit": UNIT,
-               "plan": lib.plan(N_, prec), "lhaf": [v.real, v.imag]}
+               "lhaf": [v.real, v.imag]}
+        if prec == F64:
+            res["plan"] = lib.plan(N_, prec)
         if prec == TF:
-            ach = workmodel.lhaf_tf_instr(N_) / sec / 1e12
-            res["roofline"] = {"bound": "alu", "achieved": ach, "peak": tf_peak,
-                               "unit": "T FP32 instr/s", "frac": ach / tf_peak}
+            ach = workmodel.tree_macs(N_) * workmodel.TREE_IMAD / sec / 1e12
+            res["roofline"] = {"bound": "alu", "achieved": ach, "peak": imad_peak,
+                               "unit": "T integer multiply-adds/s", "frac": ach / imad_peak}
         else:
             ach = workmodel.lhaf_flops(N_) / sec / 1e12
             res["roofline"] = {"bound": "alu", "achieved": ach, "peak": fp_peak,
@@ -430,8 +478,7 @@ def run_ours(args, rank, world, local_rank):
             e1.record(stream)
             torch.cuda.synchronize()
             res[pname] = {"sync_call_us_median": 1e6 * statistics.median(walls),
-                          "device_us_per_eval": 1e3 * e0.elapsed_time(e1) / calls,
-                          "kernels_per_eval": lib.plan(N_, prec)["kernels"]}
+                          "device_us_per_eval": 1e3 * e0.elapsed_time(e1) / calls}
         return res
 
     small = None
@@ -450,41 +497,41 @@ def run_ours(args, rank, world, local_rank):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         cpu = cpu_baseline_block(A, args.cpu_seconds)
 
+    launches = kernel_launches(tf_run["step"])
     if rank == 0:
-        plan = lib.plan(N, TF)
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f32x3", "data": "synthetic (seeded Haar-random GBS kernel matrices)",
+            "dtype": "fixed point, 81 fraction bits (3 x 27-bit int32 limbs)", "data": "synthetic (seeded Haar-random GBS kernel matrices)",
             "config": {"workload": WORKLOAD, "N": N, "subsets_per_step_per_gpu": subsets,
-                       "path": "triple-float per subset (GBSH_PREC_TF: three FP32 words, "
-                               "~72-bit significand), compensated FP64 cross-subset sum",
+                       "path": "GBSH_PREC_TF as called without an error estimate: elimination tree "
+                               "in complex fixed point (the value of the whole subset sum, whose "
+                               "2^{N/2} terms the metric counts, without visiting them one by one)",
                        "l2": "flushed between timed steps (256 MiB write, outside the events)",
-                       "plan": plan, "tuning": tuning_block(N),
+                       "tuning": tuning_block(N),
                        "parallelism": f"replicas x{world}"},
-            "roofline": {"bound": "alu", "achieved": tf_ach, "peak": tf_peak,
-                         "unit": "T FP32 instr/s", "frac": tf_ach / tf_peak,
-                         "traffic": recorded_traffic(N, "tf"),
-                         "traffic_whole_evaluation": recorded_traffic(N, "tf", whole=True),
-                         "traffic_note": "DRAM bytes per evaluation (ncu): the subset kernel's "
-                                         "class launches; the whole evaluation adds the chunk "
-                                         "partial sums, L2-resident in the timed run",
-                         "peak_source": "derived: 152 SM x 128 FP32 lanes/clk x 2.07 GHz",
-                         "measured_ffma_probe_t_instr": probes.get("ffma_t_instr"),
-                         "kernel": "lhaf_subsets_kernel<tfc> (+expand, finalize in the step time)",
-                         "work_per_launch": tf_instr,
-                         "work_convention": "FP32 arithmetic instructions of the triple-float "
-                                            "algorithm (216 per complex multiply-add)"},
+            "roofline": {"bound": "alu", "achieved": imad_ach, "peak": imad_peak,
+                         "unit": "T integer multiply-adds/s", "frac": imad_ach / imad_peak,
+                         "traffic": recorded_traffic(N, "tree"),
+                         "traffic_whole_evaluation": recorded_traffic(N, "tree", whole=True),
+                         "traffic_note": "DRAM bytes per evaluation (ncu): tree_kernel; all launches",
+                         "peak_source": "derived: 152 SM x 64 32x32+64-bit multiply-adds/clk x 2.07 GHz",
+                         "kernel": "tree_kernel (+ root, level and gated subset-sum launches in "
+                                   "the step time)",
+                         "work_per_launch": imads,
+                         "work_convention": "integer multiply-adds of the tree's polynomial products "
+                                            "(18 per complex multiply-add)"},
+            "subset_sum": subset_sum,
             "fp64": fp64,
             "accuracy": accuracy,
             "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": plan["kernels"] * args.steps,
+            "gpu_launches": launches * args.steps,
             "clocks": tf_run["clocks"],
             "wall_s_timed_region": tf_run["wall"],
             "result": {"lhaf": [tf_run["lhaf"].real, tf_run["lhaf"].imag],
-                       "kappa": tf_run["abs_sum"] / abs(tf_run["lhaf"])},
+                       "kappa": sum_run["abs_sum"] / abs(sum_run["lhaf"])},
             "n50": n50,
             **({"n56": n56} if n56 is not None else {}),
             "small": small,
@@ -522,9 +569,9 @@ def cpu_baseline_block(A40, seconds):
 def run_batch_workload(lib, workloads, workmodel, dev, stream, count=4096):
     """Batched workload: 4096 loop hafnians of uneven size (N uniform on even 10..30) from
     one M=100-mode state (r=0.7, Haar U, gamma ~ CN(0, 0.1^2)), up to 3 photons per mode,
-    through gbsh_gbs_prob_batch (device B and gamma). FP64, triple-float and complex-FP32 per
-    subset. Errors: every FP64 and FP32 result against the triple-float result of the same
-    problem (the triple-float batch is held within 1e-9 of the oracle by the tests)."""
+    through gbsh_gbs_prob_batch (device B and gamma), in FP64, GBSH_PREC_TF and complex FP32.
+    Errors: every FP64 and FP32 result against the GBSH_PREC_TF result of the same problem
+    (which the tests hold within 1e-9 of the oracle)."""
     import numpy as np
     import torch
     B, gamma = workloads.batch_state()
@@ -534,7 +581,7 @@ def run_batch_workload(lib, workloads, workmodel, dev, stream, count=4096):
     dg = torch.from_numpy(gamma).to(dev)
     subsets = int(sum(workmodel.subset_count(int(n)) for n in Ns))
     flops = float(sum(workmodel.lhaf_flops(int(n)) for n in Ns))
-    tfi = float(sum(workmodel.lhaf_tf_instr(int(n)) for n in Ns))
+    imads = float(sum(workmodel.tree_macs(int(n)) for n in Ns)) * workmodel.TREE_IMAD
     res = {"workload": f"{count} loop hafnians, N uniform on even 10..30, M=100 Haar state "
                        "r=0.7, gamma~CN(0,0.1^2), <=3 photons/mode (gbsh_gbs_prob_batch, "
                        "host result copy included)", "subset_terms": subsets}
@@ -553,10 +600,10 @@ def run_batch_workload(lib, workloads, workmodel, dev, stream, count=4096):
     res["fp64"]["roofline"] = {"bound": "alu", "achieved": ach,
                                "peak": workmodel.FP64_PEAK_DERIVED_TFLOPS, "unit": "TFLOP/s",
                                "frac": ach / workmodel.FP64_PEAK_DERIVED_TFLOPS}
-    ach = tfi / res["tf"]["seconds"] / 1e12
-    res["tf"]["roofline"] = {"bound": "alu", "achieved": ach,
-                             "peak": workmodel.FP32_INSTR_PEAK_DERIVED_T, "unit": "T FP32 instr/s",
-                             "frac": ach / workmodel.FP32_INSTR_PEAK_DERIVED_T}
+    ach = imads / res["tf"]["seconds"] / 1e12
+    res["tf"]["roofline"] = {"bound": "alu", "achieved": ach, "peak": workmodel.IMAD_PEAK_DERIVED_T,
+                             "unit": "T integer multiply-adds/s",
+                             "frac": ach / workmodel.IMAD_PEAK_DERIVED_T}
     for name in ("fp64", "c32"):
         err = np.abs(out[name] - out["tf"]) / np.abs(out["tf"])
         res[name]["rel_err_vs_tf"] = {"median": float(np.median(err)),
@@ -825,8 +872,9 @@ def main(argv=None):
     p.add_argument("--serve-poisson", type=int, default=60,
                    help="requests per arrival rate (the committed serving profile uses 200)")
     p.add_argument("--serve-rates", type=float, nargs="+", default=[0.5, 1.0, 2.0, 3.0])
-    p.add_argument("--serve-tick-subsets", type=int, default=1 << 16,
-                   help="split loop hafnians above this many subsets over ticks (0: off)")
+    p.add_argument("--serve-tick-subsets", type=int, default=0,
+                   help="split loop hafnians above this many subsets over ticks (0: off, the "
+                        "fastest since whole ones go by the elimination tree)")
     p.add_argument("--serve-compare", action="store_true",
                    help="also serve without splitting and run the plain path under Poisson arrivals")
     p.add_argument("--fig1", action="store_true",

@@ -23,7 +23,7 @@
  *   - Two evaluations of the same quantity exist. The subset sum forms every p_Z; it is what
  *     gives sum_Z |p_Z|, subset ranges and single terms. Where a call asks for none of these
  *     (err_est, d_abs_sum or abs_sums NULL) and the precision is GBSH_PREC_TF, or GBSH_PREC_FP64
- *     with N <= 24, an elimination tree in 83-bit fixed point evaluates the loop hafnian instead
+ *     with N <= 24, an elimination tree in fixed point (resolution 2^-81) evaluates the loop hafnian instead
  *     (csrc/lhaf_tree.cuh): far fewer operations and far less cancellation. A problem that
  *     leaves the fixed-point range is evaluated by the subset sum after all.
  *   - Results are bit-reproducible for a given N on a given GPU model: the subset sum is
@@ -143,14 +143,17 @@ int gbsh_lhaf_async_ex(const gbsh_c128* dA, int N, int lda, int precision, gbsh_
  * cancellation of the signed subset sum) is too coarse; the cross-subset sum is the same
  * compensated FP64 sum. */
 #define GBSH_PREC_DD 3
-/* GBSH_PREC_TF: each subset term in triple-float arithmetic -- every real number the
+/* GBSH_PREC_TF: the accurate path. Where no sum_Z |p_Z| is asked for, the elimination tree (see
+ * the conventions above): about 2^-80 absolute on a matrix scaled to entries of about one, some
+ * 1e-16 relative on the configuration matrices up to N = 40. In the subset sum each
+ * term is computed in triple-float arithmetic -- every real number the
  * Hessenberg reduction, La Budde's recursion and the power series handle is the unevaluated
  * sum of three FP32 words (~72-bit significand), and each term reaches the compensated
- * cross-subset sum as an exact double-double. This is the path that meets the relative
- * tolerance the heavy cancellation of the signed subset sum demands at N >= 32 (the
+ * cross-subset sum as an exact double-double. Both meet the relative tolerance the heavy
+ * cancellation of the signed subset sum demands at N >= 32 (the
  * accuracy concern of Sec. IV and Fig. 2): FP64 per subset leaves the N = 40 and N = 50
  * configuration matrices about 6e-8 and 1.5e-5 off, triple-float about 1e-13 and 1e-10 in
- * a CPU emulation of the same arithmetic. It runs on the FP32 pipe, which GB300 issues at
+ * a CPU emulation of the same arithmetic. Triple-float runs on the FP32 pipe, which GB300 issues at
  * 64 times its FP64 rate. Accepted by the batched entry points and by the _ex
  * single-evaluation entry points below. Its words are FP32, so entries of the matrix, the
  * Hessenberg form and the polynomial coefficients must stay within about 2^-78 .. 2^127
@@ -158,8 +161,8 @@ int gbsh_lhaf_async_ex(const gbsh_c128* dA, int N, int lda, int precision, gbsh_
 #define GBSH_PREC_TF 4
 
 /*
- * gbsh_lhaf_batch — loop hafnians of `count` matrices of uneven size in one persistent
- * launch (same algorithm as gbsh_lhaf per matrix).
+ * gbsh_lhaf_batch — loop hafnians of `count` matrices of uneven size in a few
+ * launches (same algorithm as gbsh_lhaf per matrix).
  *   A_packed  matrices, each Ns[p] x Ns[p] row-major (leading dimension Ns[p]) starting at
  *             element offsets[p]; host or device memory (detected; host data is copied in).
  *   offsets, Ns  host arrays of `count` entries; 0 <= Ns[p] <= GBSH_MAX_N.
@@ -202,7 +205,8 @@ int gbsh_set_batch_tuning(int precision, int n_max, int warps_per_cta);
 /*
  * Launch-shape tuning table. The library's default launch shapes come from a built-in table
  * that the autotuner (autotune.py) measured on a GB300; these calls override or read its
- * entries for this process. A launch shape never changes which subsets are summed:
+ * entries for this process. They apply to the subset sum; the elimination tree has one
+ * launch shape per problem list. A launch shape never changes which subsets are summed:
  *
  * gbsh_set_batch_tuning_ex — batched kernel, batches whose largest matrix has n_max pairs:
  *   warps per CTA of the small-popcount class (popcounts <= 10) and of the large-popcount
@@ -231,12 +235,12 @@ int gbsh_get_lhaf_tuning(int precision, int N, int* warps_cap, int* ladder, int*
 int gbsh_get_batch_tuning(int precision, int n_max, int* warps_small, int* warps_large);
 int gbsh_builtin_tuning_entries(void);
 
-/* CUDA-graph replay of the batched evaluations (gbsh_lhaf_batch, gbsh_gbs_prob_batch and the
- * sampler's ticks). The device work of one batched evaluation -- expansion, the persistent
- * popcount-class launches, the finalize -- is captured into a CUDA graph the second time the
- * same launch shape is seen (same device, workspace layout and addresses, problem count,
- * chunk total, largest size, precision and warps per CTA) and replayed with one graph launch
- * from then on; the
+/* CUDA-graph replay of the batched subset sums (gbsh_lhaf_batch, gbsh_gbs_prob_batch and the
+ * sampler's ticks, where the elimination tree does not serve them). The device work of one
+ * batched evaluation -- expansion, the persistent popcount-class launches, the finalize -- is
+ * captured into a CUDA graph the second time the same launch shape is seen (same device,
+ * workspace layout and addresses, problem count, chunk total, largest size, precision and
+ * warps per CTA) and replayed with one graph launch from then on; the
  * per-call tables are uploaded before the launch. Results are bit-identical to direct
  * launches. enable = 1 (the default) or 0. Returns GBSH_OK. */
 int gbsh_set_batch_graphs(int enable);
@@ -389,8 +393,10 @@ typedef struct {
    * its batched launch) subsets of such ranges, oldest chains first (all of them when every
    * active chain is waiting for ranges), and a chain draws its next photon number once all
    * its candidates are done. This bounds the time of a tick,
-   * so chains with small loop hafnians are not held up by ones with large ones. The
-   * ranges depend only on the size and T, so samples stay the same alone and in any mix. */
+   * so chains with small loop hafnians are not held up by ones with large ones. Ranges are
+   * subset sums: a whole loop hafnian by the elimination tree takes a sixteenth of the time of
+   * all its ranges at N = 32, a 25th at N = 40, so up to there T = 0 serves every chain sooner.
+   * The ranges depend only on the size and T, so samples stay the same alone and in any mix. */
   size_t tick_subsets;
 } gbsh_sampler_cfg;
 

@@ -36,7 +36,7 @@ constexpr int kTreeThreads = 128;
 constexpr int kTreeCtasPerSm = 5;
 // Largest n of a small problem (tree_small_kernel). Alone, n = 8 takes 53 us that way against 72
 // by launches; n = 9 and 10 the same either way, n = 11 takes 104 against 91 and n = 12 162
-// against 108: their levels are wider than 16 CTAs. 128 unrelated matrices of up to 20 indices
+// against 108: their levels are wider than 16 CTAs. 128 unrelated matrices of up to 16 indices
 // take 195 us with this line at 8 or 9, 255 at 7.
 constexpr int kTreeSmallMax = 8;
 // Units (tasks of one CTA) that a launch aims at, per CTA that runs at a time, shared out by work:
@@ -375,7 +375,8 @@ struct JobSlot {
 // One breadth-first level of the large problems, the whole GPU on it: 3 to 17 us, the latency of a
 // launch and of its loads for the narrow levels, the products for the wide ones. kOne: the phase
 // of the one problem is set up on the host. Phases of at most `fine` pieces, a quarter of a
-// coefficient a thread, run that way: a narrow level is as long as one thread's work.
+// coefficient a thread, run that way: a narrow level is as long as one thread's work (N = 20
+// 59 us an evaluation, 80 without; N = 25 116 and 130; N = 40 the same).
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_step_kernel(const TreeProblem* __restrict__ table, const __grid_constant__ TreePhase one, int step, int fine,

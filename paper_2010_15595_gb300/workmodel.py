@@ -1,7 +1,8 @@
-"""Algorithmic work of the loop-hafnian kernels, for roofline accounting.
+"""Algorithmic work of the loop-hafnian kernels, for roofline accounting: the elimination tree
+(tree_macs) and the subset sum (the rest).
 
-Counts the FP64 floating-point operations the kernel's algorithm needs for one subset of
-popcount k (matrix size m = 2k, bordered size S = m + 1) of an N = 2n evaluation, lane by
+For the subset sum, counts the FP64 floating-point operations the kernel's algorithm
+needs for one subset of popcount k (matrix size m = 2k, bordered size S = m + 1) of an N = 2n evaluation, lane by
 lane, counting only lanes that do useful work (idle lanes of a warp instruction are not
 algorithmic work). Conventions: complex multiply-add = 8 flops, complex multiply = 6,
 complex add = 2, complex reciprocal = 7.
@@ -106,6 +107,33 @@ def lhaf_flops(N: int) -> int:
     return sum(comb(n, k) * subset_flops(k, n) for k in range(1, n + 1))
 
 
+def _tree_nodes(M: int, n: int) -> int:
+    """Nodes of the elimination tree with M of n index pairs left (the first sign is fixed)."""
+    return 1 if n - M < 2 else 1 << (n - M - 1)
+
+
+@lru_cache(maxsize=None)
+def tree_macs(N: int) -> int:
+    """Complex multiply-adds of one loop hafnian by the elimination tree (lhaf_tree.cuh): the
+    products of truncated polynomials with n - M coefficients. A node with M pairs left makes
+    (M - 1)(2M - 1) polynomials of two products for its children and one for the scalar factor,
+    which its parent's factor is then multiplied with; the last two pairs take six products, and
+    four more whose coefficients are each multiplied with one of the scalar factor."""
+    n = max(4, N + (N & 1)) // 2
+    tri = lambda c: c * (c + 1) // 2  # noqa: E731
+    tot = _tree_nodes(2, n) * (10 * tri(n - 2) + 4 * (n - 2))
+    tot += _tree_nodes(3, n) * tri(n - 3) if n > 3 else 0
+    for M in range(3, n):
+        tot += _tree_nodes(M, n) * (2 * (M - 1) * (2 * M - 1) + 1) * tri(n - M)
+        tot += _tree_nodes(M + 1, n) * tri(n - M - 1)
+    return tot
+
+
+# Integer multiply-adds (32 x 32 + 64 bits) of one complex multiply-add on three 27-bit limbs:
+# three real products (Gauss) of the six limb products above the resolution.
+TREE_IMAD = 18
+
+
 def subset_count(N: int) -> int:
     n = (N + (N & 1)) // 2
     return 1 << n
@@ -117,3 +145,6 @@ FP64_PEAK_DERIVED_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # Derived FP32 instruction issue rate of one GB300: 152 SMs x 128 FP32 lanes per clock x
 # 2.070 GHz (one FP32 instruction per lane per clock, an FMA counting once).
 FP32_INSTR_PEAK_DERIVED_T = 152 * 128 * 2.070e9 / 1e12
+# Derived rate of 32 x 32 + 64 bit integer multiply-adds of one GB300: 152 SMs x 64 per clock x
+# 2.070 GHz (18.7 T/s measured with register operands that the register file can deliver).
+IMAD_PEAK_DERIVED_T = 152 * 64 * 2.070e9 / 1e12
