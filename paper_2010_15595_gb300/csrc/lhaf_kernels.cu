@@ -531,6 +531,13 @@ static cudaError_t side_streams(cudaStream_t** out) {
   return cudaSuccess;
 }
 
+cudaError_t side_stream(cudaStream_t* out) {
+  cudaStream_t* streams = nullptr;
+  const cudaError_t e = side_streams(&streams);
+  if (e == cudaSuccess) *out = streams[1];
+  return e;
+}
+
 // Launches every popcount class. Class 0 runs on `stream`; the others on the side streams,
 // forked from and joined back into `stream` with events, so all work of the evaluation is
 // ordered after what precedes it on `stream` and before what follows.

@@ -46,7 +46,7 @@ struct TreePlan {
   std::vector<Step> steps;         // breadth-first eliminations: problems that take part (the
                                    // first ones), most tasks of one of them
   size_t cta_bytes;                // scratch per CTA
-  size_t off_prob, off_state, off_counter, off_out, off_root, off_cta, bytes;
+  size_t off_prob, off_state, off_counter, off_out, off_root, off_cta, off_small, bytes;
 };
 
 // Sizes 0 are left out (their loop hafnian is 1): `Ns` entries must be 1..kMaxN.
