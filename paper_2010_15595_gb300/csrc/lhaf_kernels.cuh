@@ -108,7 +108,8 @@ cudaError_t launch_batch(const BatchInput* d_in, const BatchProblem* d_prob, int
                          int warps_small, unsigned* d_counter, double* d_partials, double* d_out,
                          cudaStream_t stream, cudaStream_t side_stream = nullptr);
 
-// A side stream of the current device (for work forked from a caller's stream and joined back).
+// A side stream of the current device, for work of synchronous calls that is forked from their
+// stream and joined back; never part of a stream capture.
 cudaError_t side_stream(cudaStream_t* out);
 
 // Launches `k`; if `chained`, so that its CTAs may start while the launch before it on the stream

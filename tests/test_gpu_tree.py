@@ -135,3 +135,27 @@ def test_graph_capture(gbsh):
         g.replay()
         torch.cuda.synchronize()
         assert complex(out.item()) == gbsh.lhaf(M, precision=gbsh.PREC_TF)
+
+
+def test_synchronous_batch_during_a_capture(gbsh):
+    """While a thread captures an evaluation of several launch classes, which takes the library's
+    side streams into the capture, synchronous batches of both kinds of problems go on."""
+    import torch
+    A = W.single_lhaf_mid(40)
+    mats = [W.single_lhaf_mid(N) for N in (8, 20)]
+    st = torch.cuda.Stream()
+    want = gbsh.lhaf_batch(mats, precision=gbsh.PREC_TF, stream=st)  # and everything is allocated
+    dA = _dev(A)
+    out = torch.zeros(1, dtype=torch.complex128, device="cuda")
+    ws = torch.empty(gbsh.workspace_size(40, gbsh.PREC_TF), dtype=torch.uint8, device="cuda")
+    gbsh.lhaf_async(dA, out, ws, precision=gbsh.PREC_TF)
+    ref = complex(out.item())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        gbsh.lhaf_async(dA, out, ws, precision=gbsh.PREC_TF)
+        got = gbsh.lhaf_batch(mats, precision=gbsh.PREC_TF, stream=st)
+    assert np.all(got == want)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert complex(out.item()) == ref
