@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <new>
 #include <numeric>
 
 #include <cooperative_groups.h>
@@ -587,7 +588,8 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
-cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan) {
+// Callers sit behind C entry points: no exception leaves.
+cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan) try {
   DeviceInfo dev;
   cudaError_t e = device_info(&dev);
   if (e != cudaSuccess) return e;
@@ -656,6 +658,8 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
   T.off_small = off; off = align256(off + T.small_bytes * (size_t)T.clusters);
   T.bytes = off;
   return cudaSuccess;
+} catch (const std::bad_alloc&) {
+  return cudaErrorMemoryAllocation;
 }
 
 cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st) {
@@ -744,7 +748,7 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
 }
 
 cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host, cudaStream_t st,
-                     double* out3, std::vector<int>* again) {
+                     double* out3, std::vector<int>* again) try {
   const size_t count = plan->prob.size();
   // The kernels write the results straight to page-locked memory: with a copy to pageable memory
   // instead (and the matrix of gbsh_lhaf copied from there), a call takes 75 us at N = 16, not 61.
@@ -766,6 +770,8 @@ cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host,
   }
   std::sort(again->begin(), again->end());
   return cudaSuccess;
+} catch (const std::bad_alloc&) {  // before anything is launched or after it has ended
+  return cudaErrorMemoryAllocation;
 }
 
 const unsigned* tree_flag(const TreePlan& plan, void* ws) {
