@@ -34,7 +34,7 @@
 // operands, 18.7e12/s, and every 4.4 in this code: its operand fetch is the limit.) Fixed point
 // needs a scale: the matrix is scaled by one factor such that its root-mean-fourth singular value
 // is about one, which keeps the coefficients of every matrix tried between 2^-10 and 2.5 (the
-// format holds |x| < 4).
+// format holds |x| < 4, long levels a little less: fx_limit).
 // Overflow anywhere, or a result so small that the 2^-81 resolution could show, sets a flag and
 // the caller evaluates the problem by the subset sum instead.
 //
@@ -134,8 +134,8 @@ GBSH_HD void fx_mac(FxAcc& s, const Fxc& a, const Fxc& b) {
   fx_mac1(s.t2, s.t1, s.t0, a.rh + a.ih, a.rm + a.im, a.rl + a.il, b.rh + b.ih, b.rm + b.im, b.rl + b.il);
 }
 
-// The accumulated real number rounded to the format: s2 2^27 + s1 + s0 2^-27; bad |= |x| >= 4.
-// (s2 itself holds |x| < 512: 32 products of numbers at the limit.)
+// The accumulated real number rounded to the format: s2 2^27 + s1 + s0 2^-27; bad |= |x| >= 4. s2
+// wraps at |x| = 512, so a sum is told from one below 4 as long as it is below 1020: see fx_limit.
 GBSH_HD void fx_norm1(long long s2, long long s1, long long s0, int& h, int& m, int& l, unsigned& bad) {
   const long long t = s1 + (s0 >> kLimbBits);
   l = ((int)t & kLimbMask) - kLimbHalf;
@@ -151,25 +151,40 @@ GBSH_HD Fxc fx_norm(const FxSum& s, unsigned& bad) {
   return r;
 }
 
-// (h, m, l) from limbs with carries to propagate; bad |= |x| >= 4.
-GBSH_HD void fx_carry(int xh, int xm, int xl, int& h, int& m, int& l, unsigned& bad) {
+// Largest |h| of a number that a level of L coefficients may hold. A coefficient of its products
+// is a sum of up to 2 L complex products (two factors' pairs), 4 L real ones in each part, which
+// stays below the 1020 that fx_norm1 needs if the numbers are below sqrt(255 / L): 4 up to 15
+// coefficients (N = 34), then less, 3.57 at N = 44 (where a configuration matrix was seen to reach
+// 3.31), 3.02 at N = 60. Level 2's numbers enter single products and may be as large as 4 at any length.
+GBSH_HD int fx_limit(int L) {
+  constexpr int kOne = 1 << (kTreeFrac - 2 * kLimbBits);
+  if (L <= 15) return 4 * kOne - 1;
+#ifdef __CUDA_ARCH__
+  return (int)(sqrtf(255.0f / (float)L) * (float)kOne) - 64;  // 64: roundings of the root
+#else
+  return (int)(__builtin_sqrtf(255.0f / (float)L) * (float)kOne) - 64;
+#endif
+}
+
+// (h, m, l) from limbs with carries to propagate; bad |= |h| > lim.
+GBSH_HD void fx_carry(int xh, int xm, int xl, int& h, int& m, int& l, int lim, unsigned& bad) {
   const int a = xl + kLimbHalf;
   l = (a & kLimbMask) - kLimbHalf;
   const int b = xm + kLimbHalf + (a >> kLimbBits);
   m = (b & kLimbMask) - kLimbHalf;
   h = xh + (b >> kLimbBits);
-  bad |= (unsigned)(h + (1 << 29)) >> 30;
+  bad |= (unsigned)((lim - h) | (lim + h)) >> 31;
 }
-GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, unsigned& bad) {
+GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, int lim, unsigned& bad) {
   Fxc r;
-  fx_carry(a.rh + b.rh, a.rm + b.rm, a.rl + b.rl, r.rh, r.rm, r.rl, bad);
-  fx_carry(a.ih + b.ih, a.im + b.im, a.il + b.il, r.ih, r.im, r.il, bad);
+  fx_carry(a.rh + b.rh, a.rm + b.rm, a.rl + b.rl, r.rh, r.rm, r.rl, lim, bad);
+  fx_carry(a.ih + b.ih, a.im + b.im, a.il + b.il, r.ih, r.im, r.il, lim, bad);
   return r;
 }
-GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, unsigned& bad) {
+GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, int lim, unsigned& bad) {
   Fxc r;
-  fx_carry(a.rh - b.rh, a.rm - b.rm, a.rl - b.rl, r.rh, r.rm, r.rl, bad);
-  fx_carry(a.ih - b.ih, a.im - b.im, a.il - b.il, r.ih, r.im, r.il, bad);
+  fx_carry(a.rh - b.rh, a.rm - b.rm, a.rl - b.rl, r.rh, r.rm, r.rl, lim, bad);
+  fx_carry(a.ih - b.ih, a.im - b.im, a.il - b.il, r.ih, r.im, r.il, lim, bad);
   return r;
 }
 
@@ -310,7 +325,7 @@ struct TreePhase {
   int src_bit, par_bit;  // a level walked depth first: its node is this bit of the walk's number;
                          // -1: its nodes are those of src and par
   // set by tree_ready
-  int nmain, items, tasks;
+  int nmain, items, tasks, lim;
   float inv_items, inv_node;
 };
 
@@ -322,6 +337,7 @@ GBSH_HD void tree_ready(TreePhase& s) {
   s.nmain = s.src.q * (s.kind == kTreeStep ? per + 1 : per);
   s.items = s.nmain + (s.kind == kTreeLast2 ? 0 : g);
   s.tasks = ((L + 1) / 2 + 1) / 2 * s.items;
+  s.lim = fx_limit(s.kind == kTreeStep && s.M > 3 ? L + 1 : 0);
   s.inv_items = 1.0f / (float)s.items;
   s.inv_node = 1.0f / (float)per;
 }
@@ -338,6 +354,7 @@ struct TreeJob {
   int old, so;         // kChild: the polynomial to which +- x (product) is added; kStore: (product)
   int dst, twin, sd;   // kChild: the + and the - child (or one, the - child if `neg`)
   int top, last;       // two below the number of coefficients; last coefficient of `old`
+  int lim;             // fx_limit of what is stored
   int node;
   bool neg;
 };
@@ -353,6 +370,7 @@ GBSH_HD TreeJob tree_job(const TreePhase& s, unsigned walk, int it) {
   J.sd = 0;
   J.top = L - 2;
   J.last = L - 1;
+  J.lim = s.lim;
   J.neg = false;
   J.node = 0;
   if (s.kind == kTreeLast2) {
@@ -444,8 +462,8 @@ GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& bad) {
     Fxc o{};
     if (t < J.last) o = fx_load(J.fb + J.old + (ptrdiff_t)(t + 1) * J.so);
     char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
-    if (!J.neg) fx_store(d + J.dst, fx_add(o, v, bad));
-    if (J.twin >= 0 || J.neg) fx_store(d + (J.neg ? J.dst : J.twin), fx_sub(o, v, bad));
+    if (!J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
+    if (J.twin >= 0 || J.neg) fx_store(d + (J.neg ? J.dst : J.twin), fx_sub(o, v, J.lim, bad));
     if (t == 0) {
       const Fxc c = fx_load(J.fb + J.old);
       fx_store(J.db + J.dst, c);
@@ -453,10 +471,10 @@ GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& bad) {
     }
   } else {
     char* d = J.db + (ptrdiff_t)t * J.sd;
-    fx_store(d + J.dst, fx_add(fx_load(J.fb + J.old + (ptrdiff_t)t * J.so), v, bad));
+    fx_store(d + J.dst, fx_add(fx_load(J.fb + J.old + (ptrdiff_t)t * J.so), v, J.lim, bad));
     if (J.twin >= 0) {
       const Fxc zero{};
-      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, bad), v, bad) : v);
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, bad), v, J.lim, bad) : v);
     }
   }
 }
@@ -472,18 +490,18 @@ GBSH_HD void tree_end_part(const TreeJob& J, int t, int role, const Fxc& o, cons
   if (J.end == kStore) {
     char* d = J.db + (ptrdiff_t)t * J.sd;
     if (role == 0) {
-      fx_store(d + J.dst, fx_add(o, v, bad));
+      fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
     } else if (role == 1 && J.twin >= 0) {
       const Fxc zero{};
-      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, bad), v, bad) : v);
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, bad), v, J.lim, bad) : v);
     }
     return;
   }
   char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
   if (role < 2) {
     if (role == 1 && J.twin < 0) return;
-    if (role == 0 && !J.neg) fx_store(d + J.dst, fx_add(o, v, bad));
-    else fx_store(d + (role == 0 ? J.dst : J.twin), fx_sub(o, v, bad));
+    if (role == 0 && !J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
+    else fx_store(d + (role == 0 ? J.dst : J.twin), fx_sub(o, v, J.lim, bad));
   } else if (t == 0 && (role == 2 || J.twin >= 0)) {
     fx_store(J.db + (role == 2 ? J.dst : J.twin), o);
   }
@@ -532,9 +550,10 @@ GBSH_HD void tree_put(const Slot& m, const TreeJob& J) {
   m.put(10, (int)J.end + (J.neg ? 4 : 0));
 }
 template <class Slot>
-GBSH_HD TreeJob tree_get(const Slot& m, const char* fb) {
+GBSH_HD TreeJob tree_get(const Slot& m, const char* fb, int lim) {
   TreeJob J;
   J.fb = fb;
+  J.lim = lim;
   J.db = (char*)(size_t)((unsigned long long)(unsigned)m.get(0) | (unsigned long long)(unsigned)m.get(1) << 32);
   J.old = m.get(4);
   J.so = m.get(5);
@@ -596,7 +615,7 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
         const Fxc v = fx_norm(sum, bad);
         sum = sum1;
         if (t < 0) continue;
-        const TreeJob J = tree_get(slot, fb);
+        const TreeJob J = tree_get(slot, fb, s.lim);
         if (J.end == kDot) {
           FxAcc dot = fx_acc_zero();
           fx_mac(dot, v, fx_load(fb + J.old + (ptrdiff_t)(J.last - t) * J.so));
