@@ -352,16 +352,18 @@ __device__ __forceinline__ bool tree_piece_task(const TreeJob& J, int t, int sub
     acc.s0i += __shfl_xor_sync(0xffffffffu, acc.s0i, d);
   }
   if (!active) return false;
-  const Fxc v = fx_norm(acc, bad);
+  unsigned& over = bad;  // as in tree_task
+  bad <<= 31;
+  const Fxc v = fx_norm(acc, over);
   if (J.end != kDot) {
-    tree_end_part(J, t, sub, old, v, bad);
-    return false;
+    tree_end_part(J, t, sub, old, v, over);
+  } else if (sub == 0) {
+    FxAcc dot = fx_acc_zero();
+    fx_mac(dot, v, old);
+    z = fx_norm(fx_sum(dot), over);
   }
-  if (sub != 0) return false;
-  FxAcc dot = fx_acc_zero();
-  fx_mac(dot, v, old);
-  z = fx_norm(fx_sum(dot), bad);
-  return true;
+  bad >>= 31;
+  return J.end == kDot && sub == 0;
 }
 
 // Column of a thread in its CTA's job storage (tree_put). Volatile: the compiler would keep the

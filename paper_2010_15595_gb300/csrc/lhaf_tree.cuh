@@ -134,20 +134,26 @@ GBSH_HD void fx_mac(FxAcc& s, const Fxc& a, const Fxc& b) {
   fx_mac1(s.t2, s.t1, s.t0, a.rh + a.ih, a.rm + a.im, a.rl + a.il, b.rh + b.ih, b.rm + b.im, b.rl + b.il);
 }
 
-// The accumulated real number rounded to the format: s2 2^27 + s1 + s0 2^-27; bad |= |x| >= 4. s2
+// Range checks set the sign bit of `over`: three instructions each, and they run on every number
+// (with the limit in a register N = 32 takes 1 % longer than with a constant 4, N = 44 4 % less).
+GBSH_HD void fx_check(int h, int lim, unsigned& over) {
+  over |= ((unsigned)lim - (unsigned)h) | ((unsigned)lim + (unsigned)h);  // |h| > lim
+}
+
+// The accumulated real number rounded to the format: s2 2^27 + s1 + s0 2^-27; `over` if |x| >= 4. s2
 // wraps at |x| = 512, so a sum is told from one below 4 as long as it is below 1020: see fx_limit.
-GBSH_HD void fx_norm1(long long s2, long long s1, long long s0, int& h, int& m, int& l, unsigned& bad) {
+GBSH_HD void fx_norm1(long long s2, long long s1, long long s0, int& h, int& m, int& l, unsigned& over) {
   const long long t = s1 + (s0 >> kLimbBits);
   l = ((int)t & kLimbMask) - kLimbHalf;
   const long long v = s2 + (t >> kLimbBits);
   m = ((int)v & kLimbMask) - kLimbHalf;
   h = (int)(v >> kLimbBits);
-  bad |= (unsigned)((int)(v >> 32) + (1 << 24)) >> 25;
+  fx_check((int)(v >> 32), (1 << 24) - 1, over);
 }
-GBSH_HD Fxc fx_norm(const FxSum& s, unsigned& bad) {
+GBSH_HD Fxc fx_norm(const FxSum& s, unsigned& over) {
   Fxc r;
-  fx_norm1(s.s2r, s.s1r, s.s0r, r.rh, r.rm, r.rl, bad);
-  fx_norm1(s.s2i, s.s1i, s.s0i, r.ih, r.im, r.il, bad);
+  fx_norm1(s.s2r, s.s1r, s.s0r, r.rh, r.rm, r.rl, over);
+  fx_norm1(s.s2i, s.s1i, s.s0i, r.ih, r.im, r.il, over);
   return r;
 }
 
@@ -166,25 +172,25 @@ GBSH_HD int fx_limit(int L) {
 #endif
 }
 
-// (h, m, l) from limbs with carries to propagate; bad |= |h| > lim.
-GBSH_HD void fx_carry(int xh, int xm, int xl, int& h, int& m, int& l, int lim, unsigned& bad) {
+// (h, m, l) from limbs with carries to propagate; `over` if |h| > lim.
+GBSH_HD void fx_carry(int xh, int xm, int xl, int& h, int& m, int& l, int lim, unsigned& over) {
   const int a = xl + kLimbHalf;
   l = (a & kLimbMask) - kLimbHalf;
   const int b = xm + kLimbHalf + (a >> kLimbBits);
   m = (b & kLimbMask) - kLimbHalf;
   h = xh + (b >> kLimbBits);
-  bad |= (unsigned)((lim - h) | (lim + h)) >> 31;
+  fx_check(h, lim, over);
 }
-GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, int lim, unsigned& bad) {
+GBSH_HD Fxc fx_add(const Fxc& a, const Fxc& b, int lim, unsigned& over) {
   Fxc r;
-  fx_carry(a.rh + b.rh, a.rm + b.rm, a.rl + b.rl, r.rh, r.rm, r.rl, lim, bad);
-  fx_carry(a.ih + b.ih, a.im + b.im, a.il + b.il, r.ih, r.im, r.il, lim, bad);
+  fx_carry(a.rh + b.rh, a.rm + b.rm, a.rl + b.rl, r.rh, r.rm, r.rl, lim, over);
+  fx_carry(a.ih + b.ih, a.im + b.im, a.il + b.il, r.ih, r.im, r.il, lim, over);
   return r;
 }
-GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, int lim, unsigned& bad) {
+GBSH_HD Fxc fx_sub(const Fxc& a, const Fxc& b, int lim, unsigned& over) {
   Fxc r;
-  fx_carry(a.rh - b.rh, a.rm - b.rm, a.rl - b.rl, r.rh, r.rm, r.rl, lim, bad);
-  fx_carry(a.ih - b.ih, a.im - b.im, a.il - b.il, r.ih, r.im, r.il, lim, bad);
+  fx_carry(a.rh - b.rh, a.rm - b.rm, a.rl - b.rl, r.rh, r.rm, r.rl, lim, over);
+  fx_carry(a.ih - b.ih, a.im - b.im, a.il - b.il, r.ih, r.im, r.il, lim, over);
   return r;
 }
 
@@ -457,13 +463,13 @@ GBSH_HD TreeJob tree_job(const TreePhase& s, unsigned walk, int it) {
 }
 
 // What becomes of coefficient t of the product.
-GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& bad) {
+GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& over) {
   if (J.end == kChild) {
     Fxc o{};
     if (t < J.last) o = fx_load(J.fb + J.old + (ptrdiff_t)(t + 1) * J.so);
     char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
-    if (!J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
-    if (J.twin >= 0 || J.neg) fx_store(d + (J.neg ? J.dst : J.twin), fx_sub(o, v, J.lim, bad));
+    if (!J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, over));
+    if (J.twin >= 0 || J.neg) fx_store(d + (J.neg ? J.dst : J.twin), fx_sub(o, v, J.lim, over));
     if (t == 0) {
       const Fxc c = fx_load(J.fb + J.old);
       fx_store(J.db + J.dst, c);
@@ -471,10 +477,10 @@ GBSH_HD void tree_end(const TreeJob& J, int t, const Fxc& v, unsigned& bad) {
     }
   } else {
     char* d = J.db + (ptrdiff_t)t * J.sd;
-    fx_store(d + J.dst, fx_add(fx_load(J.fb + J.old + (ptrdiff_t)t * J.so), v, J.lim, bad));
+    fx_store(d + J.dst, fx_add(fx_load(J.fb + J.old + (ptrdiff_t)t * J.so), v, J.lim, over));
     if (J.twin >= 0) {
       const Fxc zero{};
-      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, bad), v, J.lim, bad) : v);
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, over), v, J.lim, over) : v);
     }
   }
 }
@@ -486,22 +492,22 @@ GBSH_HD Fxc tree_end_old(const TreeJob& J, int t, int role) {
   if (role < 2) return t < J.last ? fx_load(J.fb + J.old + (ptrdiff_t)(t + 1) * J.so) : Fxc{};
   return t == 0 ? fx_load(J.fb + J.old) : Fxc{};
 }
-GBSH_HD void tree_end_part(const TreeJob& J, int t, int role, const Fxc& o, const Fxc& v, unsigned& bad) {
+GBSH_HD void tree_end_part(const TreeJob& J, int t, int role, const Fxc& o, const Fxc& v, unsigned& over) {
   if (J.end == kStore) {
     char* d = J.db + (ptrdiff_t)t * J.sd;
     if (role == 0) {
-      fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
+      fx_store(d + J.dst, fx_add(o, v, J.lim, over));
     } else if (role == 1 && J.twin >= 0) {
       const Fxc zero{};
-      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, bad), v, J.lim, bad) : v);
+      fx_store(d + J.twin, J.neg ? fx_sub(fx_sub(zero, v, J.lim, over), v, J.lim, over) : v);
     }
     return;
   }
   char* d = J.db + (ptrdiff_t)(t + 1) * J.sd;
   if (role < 2) {
     if (role == 1 && J.twin < 0) return;
-    if (role == 0 && !J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, bad));
-    else fx_store(d + (role == 0 ? J.dst : J.twin), fx_sub(o, v, J.lim, bad));
+    if (role == 0 && !J.neg) fx_store(d + J.dst, fx_add(o, v, J.lim, over));
+    else fx_store(d + (role == 0 ? J.dst : J.twin), fx_sub(o, v, J.lim, over));
   } else if (t == 0 && (role == 2 || J.twin >= 0)) {
     fx_store(J.db + (role == 2 ? J.dst : J.twin), o);
   }
@@ -569,7 +575,7 @@ GBSH_HD TreeJob tree_get(const Slot& m, const char* fb, int lim) {
 }
 
 // Runs one task of walk `walk`. In phase last2 returns true with a part of node `node`'s term in
-// z (sums of limbs, carries not propagated).
+// z (sums of limbs, carries not propagated). bad: 0, or 1 once a number left the range.
 template <class Slot>
 GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& slot, int& node, Fxc& z,
                        unsigned& bad) {
@@ -588,6 +594,8 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
     top = J.top;
   }
   z = Fxc{};
+  unsigned& over = bad;  // one register: the sign bit until the end of the task
+  bad <<= 31;
 #ifdef __CUDA_ARCH__
 #pragma unroll 1
 #endif
@@ -612,17 +620,17 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
 #pragma unroll 1
 #endif
       for (int t = t0; t < t0 + 2; ++t) {
-        const Fxc v = fx_norm(sum, bad);
+        const Fxc v = fx_norm(sum, over);
         sum = sum1;
         if (t < 0) continue;
         const TreeJob J = tree_get(slot, fb, s.lim);
         if (J.end == kDot) {
           FxAcc dot = fx_acc_zero();
           fx_mac(dot, v, fx_load(fb + J.old + (ptrdiff_t)(J.last - t) * J.so));
-          const Fxc part = fx_norm(fx_sum(dot), bad);
+          const Fxc part = fx_norm(fx_sum(dot), over);
           z = Fxc{z.rh + part.rh, z.rm + part.rm, z.rl + part.rl, z.ih + part.ih, z.im + part.im, z.il + part.il};
         } else {
-          tree_end(J, t, v, bad);
+          tree_end(J, t, v, over);
         }
       }
     }
@@ -630,6 +638,7 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
     if (side == 1 || mirror == tile) break;
     tile = mirror;
   }
+  bad >>= 31;
   return s.kind == kTreeLast2;
 }
 
