@@ -49,6 +49,7 @@ struct Scratch {
   void* ptr = nullptr;
   size_t bytes = 0;
   char* host = nullptr;
+  cudaStream_t side = nullptr;  // where a call's work forks to; never part of a stream capture
 };
 Scratch g_scratch[64];
 
@@ -79,6 +80,15 @@ char* scratch_host(Scratch& s) {
     s.host = nullptr;
   }
   return s.host;
+}
+
+// The side stream, or null where there is none.
+cudaStream_t scratch_side(Scratch& s) {
+  if (!s.side && cudaStreamCreateWithFlags(&s.side, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    s.side = nullptr;
+  }
+  return s.side;
 }
 
 cudaMemoryType memory_type(const void* p) {
@@ -165,7 +175,7 @@ int tree_sync(gbsh::TreePlan* tp, const gbsh::BatchInput& in, void* ws, void* ho
               gbsh_c128* out, bool* done) {
   double res[3];
   std::vector<int> again;
-  GBSH_CUDA(gbsh::tree_run(tp, &in, ws, host, st, res, &again));
+  GBSH_CUDA(gbsh::tree_run(tp, &in, ws, host, st, nullptr, res, &again));
   *done = again.empty();
   if (*done) {
     out->re = res[0];
@@ -244,7 +254,7 @@ int batch_plan(const int* Ns, int count, int precision, bool want_abs, size_t st
 // evaluates the problems with N <= GBSH_C32_MAX_N in complex FP32, the others as FP64), then by
 // the subset sum what the tree hands back.
 int batch_run_planned(BatchPlan* B, const int* Ns, const std::vector<gbsh::BatchInput>& in, int count,
-                      size_t staged, void* ws, void* host, cudaStream_t st, double* out3) {
+                      size_t staged, void* ws, void* host, cudaStream_t st, cudaStream_t side, double* out3) {
   if ((int)B->rest.size() == count) return batch_run(B->L, in, count, B->rest_prec, ws, st, out3);
   std::vector<int> again;
   if (!B->tree.empty()) {
@@ -252,7 +262,7 @@ int batch_run_planned(BatchPlan* B, const int* Ns, const std::vector<gbsh::Batch
     std::vector<double> o((size_t)3 * B->tree.size());
     for (size_t q = 0; q < B->tree.size(); ++q) in_sel[q] = in[B->tree[q]];
     GBSH_CUDA(gbsh::tree_run(&B->T, in_sel.data(), ws, sizeof(double) * o.size() <= kHostInput ? host : nullptr,
-                             st, o.data(), &again));
+                             st, side, o.data(), &again));
     for (size_t q = 0; q < B->tree.size(); ++q)
       for (int j = 0; j < 3; ++j) out3[3 * (size_t)B->tree[q] + j] = o[3 * q + j];
     for (int& p : again) p = B->tree[p];
@@ -420,7 +430,7 @@ int gbsh_lhaf_async_ex(const gbsh_c128* dA, int N, int lda, int precision, gbsh_
     double* value = reinterpret_cast<double*>(d_out);
     const gbsh::BatchInput in{reinterpret_cast<const double2*>(dA), nullptr, nullptr, lda, N};
     GBSH_CUDA(gbsh::tree_stage(&tp, &in, workspace, st));
-    GBSH_CUDA(gbsh::tree_launch(tp, workspace, st, value, false));
+    GBSH_CUDA(gbsh::tree_launch(tp, workspace, st, nullptr, value, false));
     GBSH_CUDA(gbsh::launch_range(plan, in.base, lda, nullptr, nullptr, workspace, st, 0,
                                  (uint64_t)1 << plan.n, gbsh::tree_flag(tp, workspace), value));
     return GBSH_OK;
@@ -625,7 +635,7 @@ int gbsh_lhaf_batch(const gbsh_c128* A_packed, const int64_t* offsets, const int
   std::vector<gbsh::BatchInput> in(count);
   for (int p = 0; p < count; ++p) in[p] = gbsh::BatchInput{base + offsets[p], nullptr, nullptr, Ns[p], Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_planned(&B, Ns, in, count, in_bytes, ws, scratch_host(s), st, out3.data());
+  rc = batch_run_planned(&B, Ns, in, count, in_bytes, ws, scratch_host(s), st, scratch_side(s), out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     outs[p].re = out3[3 * p];
@@ -704,7 +714,7 @@ int gbsh_gbs_prob_batch(const gbsh_c128* B, int M, int ldb, const gbsh_c128* gam
   for (int p = 0; p < count; ++p)
     in[p] = gbsh::BatchInput{dB, dg + gstride * p, d_idx + idx_off[p], ld, Ns[p]};
   std::vector<double> out3(3 * (size_t)count);
-  rc = batch_run_planned(&plan, Ns.data(), in, count, staged, ws, scratch_host(s), st, out3.data());
+  rc = batch_run_planned(&plan, Ns.data(), in, count, staged, ws, scratch_host(s), st, scratch_side(s), out3.data());
   if (rc != GBSH_OK) return rc;
   for (int p = 0; p < count; ++p) {
     const double re = out3[3 * p], im = out3[3 * p + 1];

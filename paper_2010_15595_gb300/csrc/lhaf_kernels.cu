@@ -508,9 +508,7 @@ static cudaError_t launch_expand(const LhafPlan& plan, const double2* base, int 
 
 // Side streams on which the popcount classes after the first run, so that the tail of one
 // class launch overlaps the next (each class has its own counter and partial sums). One set
-// per device, created on first use and kept for the life of the process. A caller that captures
-// an asynchronous evaluation takes streams 1 and up into its capture for a while; stream 0 is
-// used by synchronous calls only, so that they can go on meanwhile in other threads.
+// per device, created on first use and kept for the life of the process.
 static cudaError_t side_streams(cudaStream_t** out) {
   static cudaStream_t streams[64][kMaxClasses] = {};
   static bool made[64] = {};
@@ -520,10 +518,10 @@ static cudaError_t side_streams(cudaStream_t** out) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_mu);
   if (!made[dev]) {
-    for (int c = 0; c < kMaxClasses; ++c) {
+    for (int c = 1; c < kMaxClasses; ++c) {
       e = cudaStreamCreateWithFlags(&streams[dev][c], cudaStreamNonBlocking);
       if (e != cudaSuccess) {
-        for (int d = 0; d < c; ++d) cudaStreamDestroy(streams[dev][d]);
+        for (int d = 1; d < c; ++d) cudaStreamDestroy(streams[dev][d]);
         return e;
       }
     }
@@ -531,13 +529,6 @@ static cudaError_t side_streams(cudaStream_t** out) {
   }
   *out = streams[dev];
   return cudaSuccess;
-}
-
-cudaError_t side_stream(cudaStream_t* out) {
-  cudaStream_t* streams = nullptr;
-  const cudaError_t e = side_streams(&streams);
-  if (e == cudaSuccess) *out = streams[0];
-  return e;
 }
 
 // Launches every popcount class. Class 0 runs on `stream`; the others on the side streams,

@@ -108,10 +108,6 @@ cudaError_t launch_batch(const BatchInput* d_in, const BatchProblem* d_prob, int
                          int warps_small, unsigned* d_counter, double* d_partials, double* d_out,
                          cudaStream_t stream, cudaStream_t side_stream = nullptr);
 
-// A side stream of the current device, for work of synchronous calls that is forked from their
-// stream and joined back; never part of a stream capture.
-cudaError_t side_stream(cudaStream_t* out);
-
 // Launches `k`; if `chained`, so that its CTAs may start while the launch before it on the stream
 // ends: the kernel itself waits for that one's results (chain_wait). Only directly after a kernel
 // of this library that was launched the plain way or waits in the same manner.

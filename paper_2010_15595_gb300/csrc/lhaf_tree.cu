@@ -722,7 +722,7 @@ static cudaError_t launch_large(const TreePlan& plan, char* b, cudaStream_t st, 
                         plan.cta_bytes, out, flags);
 }
 
-cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* out, bool flags) {
+cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, cudaStream_t side, double* out, bool flags) {
   const int count = (int)plan.prob.size();
   char* b = static_cast<char*>(ws);
   if (count == 0) return cudaSuccess;
@@ -730,10 +730,12 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
   if (plan.nbig == count) return launch_large(plan, b, st, out, flags);
   // Both kinds: chains of dependent steps that leave most of the GPU idle, so side by side (a
   // sampler run of 16 samples, 40 modes, 3.18 ms; 3.70 one after the other).
-  cudaStream_t side = nullptr;
+  if (!side) {
+    const cudaError_t e = launch_small(plan, b, st, out, flags);
+    return e == cudaSuccess ? launch_large(plan, b, st, out, flags) : e;
+  }
   cudaEvent_t fork = nullptr, join = nullptr;
-  cudaError_t e = side_stream(&side);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+  cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventRecord(fork, st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
@@ -750,7 +752,7 @@ cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double*
 }
 
 cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host, cudaStream_t st,
-                     double* out3, std::vector<int>* again) try {
+                     cudaStream_t side, double* out3, std::vector<int>* again) try {
   const size_t count = plan->prob.size();
   // The kernels write the results straight to page-locked memory: with a copy to pageable memory
   // instead (and the matrix of gbsh_lhaf copied from there), a call takes 75 us at N = 16, not 61.
@@ -758,7 +760,7 @@ cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host,
   double* res = host ? static_cast<double*>(host) : pageable.data();
   double* out = host ? res : reinterpret_cast<double*>(static_cast<char*>(ws) + plan->off_out);
   cudaError_t e = tree_stage(plan, in, ws, st);
-  if (e == cudaSuccess) e = tree_launch(*plan, ws, st, out, true);
+  if (e == cudaSuccess) e = tree_launch(*plan, ws, st, side, out, true);
   if (e == cudaSuccess && !host && count > 0)
     e = cudaMemcpyAsync(res, out, sizeof(double) * 3 * count, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

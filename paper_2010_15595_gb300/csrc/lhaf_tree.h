@@ -52,11 +52,13 @@ struct TreePlan {
 // Sizes 0 are left out (their loop hafnian is 1): `Ns` entries must be 1..kMaxN.
 cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan);
 
-// Evaluates the problems of `plan` (in[i]: input of the caller's problem i) in `ws` on `st`.
+// Evaluates the problems of `plan` (in[i]: input of the caller's problem i) in `ws` on `st`. `side`: a
+// stream that nothing else uses until `st` has been waited for, to which part of the work may be
+// forked from `st` and joined back, or null.
 // Result of launch-order problem q, if `flags`: three doubles at out + 3 q: re, im, and 1 where
 // the problem has to be evaluated by the subset sum instead (0 otherwise). Without (one-problem
 // launches): re, im, and the flag at tree_flag().
-cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, double* out, bool flags);
+cudaError_t tree_launch(const TreePlan& plan, void* ws, cudaStream_t st, cudaStream_t side, double* out, bool flags);
 
 // Fills in the inputs and, for more than one problem, uploads the table.
 cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStream_t st);
@@ -65,7 +67,7 @@ cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStrea
 // problem i (re, im, 0); problems to be evaluated by the subset sum are added to `again`.
 // `host`: page-locked memory of at least 24 bytes a problem that the call may use, or null.
 cudaError_t tree_run(TreePlan* plan, const BatchInput* in, void* ws, void* host, cudaStream_t st,
-                     double* out3, std::vector<int>* again);
+                     cudaStream_t side, double* out3, std::vector<int>* again);
 
 // Device address of a one-problem launch's fallback flag (nonzero: evaluate by the subset sum).
 const unsigned* tree_flag(const TreePlan& plan, void* ws);

@@ -212,7 +212,7 @@ struct gbsh_sampler {
   std::deque<Chain> pending;
   Clock::time_point t0 = Clock::now();
   // device state (worker thread only)
-  cudaStream_t st = nullptr;
+  cudaStream_t st = nullptr, side = nullptr;
   double2 *dB = nullptr, *dgbar = nullptr, *dalpha = nullptr, *dgam = nullptr;
   int *dslot = nullptr, *dk = nullptr, *didx = nullptr;
   size_t idx_cap = 0;
@@ -414,7 +414,7 @@ int gbsh_sampler::tick(std::vector<Chain>& active) {
       for (size_t q = 0; q < m; ++q) some[q] = in[sel[f + q]];
       std::vector<double> o(3 * m);
       std::vector<int> again;
-      e = gbsh::tree_run(&T, some.data(), ws, sizeof(double) * o.size() <= kHostBytes ? host : nullptr, st,
+      e = gbsh::tree_run(&T, some.data(), ws, sizeof(double) * o.size() <= kHostBytes ? host : nullptr, st, side,
                          o.data(), &again);
       if (e != cudaSuccess) return from_cuda(e);
       for (size_t q = 0; q < m; ++q)
@@ -794,6 +794,10 @@ int gbsh_sampler_create(const gbsh_sampler_cfg* cfg, gbsh_sampler** out) {
     cudaGetLastError();
     h->host = nullptr;
   }
+  if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    h->side = nullptr;
+  }
   cudaSetDevice(prev);
   gbsh_sampler* raw = h.release();
   raw->worker = std::thread([raw] { raw->run(); });
@@ -907,6 +911,7 @@ int gbsh_sampler_destroy(gbsh_sampler* h) {
   cudaFree(h->ws);
   cudaFreeHost(h->host);
   if (h->st) cudaStreamDestroy(h->st);
+  if (h->side) cudaStreamDestroy(h->side);
   cudaSetDevice(prev);
   delete h;
   return GBSH_OK;
