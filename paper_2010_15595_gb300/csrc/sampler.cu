@@ -222,6 +222,7 @@ struct gbsh_sampler {
   double* dpart = nullptr;  // range partials of one tick (5 doubles each)
   size_t part_cap = 0;
   std::vector<int> free_slots;
+  int tree_n = 0;  // largest loop hafnian that the elimination tree evaluates within mem_budget
 
   void run();
   int tick(std::vector<Chain>& active);
@@ -262,7 +263,11 @@ int gbsh_sampler::ensure_ws(size_t bytes) {
   ws_bytes = 0;
   size_t want = std::max(bytes, (size_t)1 << 22);
   cudaError_t e = cudaMalloc(&ws, want);
-  if (e != cudaSuccess) return from_cuda(e);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // the caller may go on with less
+    ws = nullptr;
+    return from_cuda(e);
+  }
   ws_bytes = want;
   return GBSH_OK;
 }
@@ -387,28 +392,40 @@ int gbsh_sampler::tick(std::vector<Chain>& active) {
                              didx + cands[q].idx_off, M, cands[q].N};
   }
   // FP64 loop hafnians of the candidates by the elimination tree (lhaf_tree.cuh; sums of exact
-  // integers, so a candidate's value is the same alone and in any mix); the complex-FP32 variant,
-  // and what the tree hands back, by the subset sum.
+  // integers, so a candidate's value is the same alone and in any mix) as far as the memory budget
+  // goes; the complex-FP32 variant, and what the tree hands back, by the subset sum.
   std::vector<int> rest;
   if (cfg.precision == GBSH_PREC_FP64) {
     std::vector<int> sel, n;
     for (int q = 0; q < nc; ++q) {
-      if (Ns[q] > 0) {
+      if (Ns[q] > tree_n) {
+        rest.push_back(q);
+      } else if (Ns[q] > 0) {
         sel.push_back(q);
         n.push_back(Ns[q]);
       } else {
         out3[3 * (size_t)q] = 1.0;
       }
     }
-    // batching: all candidates in one launch; plain path: one launch sequence and one
-    // synchronisation per candidate, what a caller of gbsh_gbs_prob would do
-    const size_t step = cfg.batching ? std::max<size_t>(sel.size(), 1) : 1;
-    for (size_t f = 0; f < sel.size(); f += step) {
-      const size_t m = std::min(step, sel.size() - f);
+    // batching: all candidates in one launch, or in as few as the memory budget (and the memory
+    // there is) allows; plain path: one launch sequence and one synchronisation per candidate,
+    // what a caller of gbsh_gbs_prob would do
+    size_t step = cfg.batching ? std::max<size_t>(sel.size(), 1) : 1, m;
+    for (size_t f = 0; f < sel.size(); f += m) {
+      m = std::min(step, sel.size() - f);
       gbsh::TreePlan T;
       e = gbsh::tree_plan(n.data() + f, (int)m, 0, &T);
       if (e != cudaSuccess) return from_cuda(e);
-      rc = ensure_ws(T.bytes);
+      rc = m > 1 && T.bytes > cfg.mem_budget ? GBSH_ENOMEM : ensure_ws(T.bytes);
+      if (rc == GBSH_ENOMEM) {
+        if (m > 1) {
+          step = (m + 1) / 2;
+          m = 0;
+        } else {
+          rest.push_back(sel[f]);
+        }
+        continue;
+      }
       if (rc != GBSH_OK) return rc;
       std::vector<gbsh::BatchInput> some(m);
       for (size_t q = 0; q < m; ++q) some[q] = in[sel[f + q]];
@@ -797,6 +814,12 @@ int gbsh_sampler_create(const gbsh_sampler_cfg* cfg, gbsh_sampler** out) {
   if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     h->side = nullptr;
+  }
+  for (int N = 1; N <= h->cfg.n_cap; ++N) {
+    gbsh::TreePlan T;
+    if ((e = gbsh::tree_plan(&N, 1, 0, &T)) != cudaSuccess) return fail(e);
+    if (T.bytes > h->cfg.mem_budget) break;
+    h->tree_n = N;
   }
   cudaSetDevice(prev);
   gbsh_sampler* raw = h.release();
