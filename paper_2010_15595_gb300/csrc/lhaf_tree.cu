@@ -588,6 +588,50 @@ constexpr int kMaxGridY = 65535;
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+using SmallKernel = void (*)(const TreeProblem*, TreeProblem, int, int, TreeState*, char*, size_t, double*, bool);
+
+static cudaLaunchConfig_t small_config(int cluster, int clusters, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(clusters * cluster));
+  cfg.blockDim = dim3(kRootThreads);
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cluster;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// CTAs of tree_small_kernel's largest cluster on the current device: 16 is not a portable size, and
+// a partition of the device may hold fewer. Asked once a device.
+static cudaError_t max_cluster(int* out) {
+  static std::mutex mu;
+  static int most[64] = {};
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!most[dev]) {
+    int c = 16;
+    for (; c > 1; c >>= 1) {
+      bool fits = true;
+      for (const SmallKernel k : {tree_small_kernel<true>, tree_small_kernel<false>}) {
+        cudaLaunchAttribute attr{};
+        const cudaLaunchConfig_t cfg = small_config(c, 1, &attr);
+        int n = 0;
+        fits = fits && (c <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+               cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n > 0;
+      }
+      if (fits) break;
+      cudaGetLastError();
+    }
+    most[dev] = c;
+  }
+  *out = most[dev];
+  return cudaSuccess;
+}
+
 }  // namespace
 
 // Callers sit behind C entry points: no exception leaves.
@@ -611,10 +655,11 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
   T.cluster = T.clusters = 0;
   T.small_bytes = 0;
   if (nsmall > 0) {
-    // CTAs that the widest levels of the largest one can use, and that the GPU has
-    const int n = pairs(T.nbig);
-    T.cluster = n <= 3 ? 1 : (n <= 4 ? 4 : (n <= 6 ? 8 : 16));
-    while (T.cluster > 1 && nsmall * T.cluster > cluster_slots) T.cluster >>= 1;
+    const int n = pairs(T.nbig);  // of the largest
+    int most = 1;
+    e = max_cluster(&most);
+    if (e != cudaSuccess) return e;
+    T.cluster = tree_cluster(n, nsmall, cluster_slots, most);
     T.clusters = std::min(nsmall, cluster_slots / T.cluster);
     T.small_bytes = align256(tree_offset(1, n));
   }
@@ -674,21 +719,10 @@ cudaError_t tree_stage(TreePlan* plan, const BatchInput* in, void* ws, cudaStrea
 static cudaError_t launch_small(const TreePlan& plan, char* b, cudaStream_t st, double* out, bool flags) {
   const int count = (int)plan.prob.size();
   const bool one = count == 1;
-  const auto k = one ? tree_small_kernel<true> : tree_small_kernel<false>;
-  if (plan.cluster > 8) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(plan.clusters * plan.cluster));
-  cfg.blockDim = dim3(kRootThreads);
-  cfg.stream = st;
+  const SmallKernel k = one ? tree_small_kernel<true> : tree_small_kernel<false>;
   cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)plan.cluster;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchConfig_t cfg = small_config(plan.cluster, plan.clusters, &attr);
+  cfg.stream = st;
   const TreeProblem* table = one ? nullptr : reinterpret_cast<const TreeProblem*>(b + plan.off_prob);
   return cudaLaunchKernelEx(&cfg, k, table, plan.prob[0], plan.nbig, count - plan.nbig,
                             reinterpret_cast<TreeState*>(b + plan.off_state), b + plan.off_small,

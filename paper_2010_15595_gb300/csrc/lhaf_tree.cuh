@@ -662,6 +662,15 @@ GBSH_HD TreePhase tree_whole_phase(char* base, int n, int i) {
   return s;
 }
 
+// CTAs of a cluster that works off whole trees of n pairs, of `count` problems: as many as the widest
+// levels can use, at most `most` (what the device can hold), and so few that `count` clusters
+// need no more than `slots` CTAs.
+GBSH_HD int tree_cluster(int n, int count, int slots, int most) {
+  int c = n <= 3 ? 1 : (n <= 4 ? 4 : (n <= 6 ? 8 : 16));
+  while (c > 1 && (c > most || (long long)count * c > slots)) c >>= 1;
+  return c;
+}
+
 // A unit: node `unit` of level m1 and all below it, in scratch of tree_scratch bytes. Levels
 // m1 - 1 .. top are walked depth first and hold the two children of one node each; from level
 // `top` on the subtree is worked off breadth first.

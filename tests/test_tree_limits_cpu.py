@@ -1,6 +1,7 @@
 """Overflow of the elimination tree's sums (csrc/lhaf_tree.cuh, built for the host). A sum of
 products is accumulated modulo 1024, so one that ends near a multiple of it would pass for a small
-number; what a level may hold is limited such that no sum of its products gets there."""
+number; what a level may hold is limited such that no sum of its products gets there. And the cluster
+sizes of the small problems."""
 import ctypes
 import math
 import os
@@ -14,12 +15,15 @@ CSRC = os.path.join(os.path.dirname(HERE), "paper_2010_15595_gb300", "csrc")
 
 
 @pytest.fixture(scope="module")
-def step(tmp_path_factory):
+def host(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("phase") / "tree_phase_host.so")
     subprocess.run(["g++", "-O2", "-std=c++17", "-fwrapv", "-shared", "-fPIC", "-I", CSRC,
                     os.path.join(HERE, "tree_phase_host.cpp"), "-o", so], check=True)
-    lib = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
 
+
+@pytest.fixture(scope="module")
+def step(host):
     def run(n, M, polys):
         """polys: {pair (j, k): coefficients}; the + child's polynomial of pair (0, 1), and the flag."""
         L, P, Pc = n - M + 1, M * (2 * M + 1), (M - 1) * (2 * M - 1)
@@ -28,7 +32,7 @@ def step(tmp_path_factory):
             src[:, k * (k - 1) // 2 + j] = c
         dst = np.zeros((L + 1, Pc), complex)
         vp = ctypes.c_void_p
-        bad = lib.tree_host_step(n, M, vp(src.ctypes.data), vp(dst.ctypes.data))
+        bad = host.tree_host_step(n, M, vp(src.ctypes.data), vp(dst.ctypes.data))
         return dst[:, 0], bad
 
     return run
@@ -83,3 +87,14 @@ def test_flags_at_the_limit_of_short_levels(step):
             old = np.full(n - M + 1, x)
             old[0] = 0.5
             assert step(n, M, {(0, 1): old})[1] == want
+
+
+@pytest.mark.parametrize("most", [1, 2, 4, 8, 16])
+def test_clusters_that_the_device_can_hold(host, most):
+    for slots in (2, 64, 304):
+        for n in range(2, 9):
+            for count in (1, 2, 5, 19, 38, 100, 1000, 2**31 // 16 + 1):
+                c = host.tree_host_cluster(n, count, slots, most)
+                assert 1 <= c <= most and c & (c - 1) == 0
+                assert c == 1 or c * count <= slots
+    assert host.tree_host_cluster(8, 1, 304, most) == most

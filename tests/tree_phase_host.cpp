@@ -1,5 +1,5 @@
-// Host build of one elimination step (csrc/lhaf_tree.cuh) on a level that the caller fills. C
-// entry for ctypes.
+// Host build of one elimination step (csrc/lhaf_tree.cuh) on a level that the caller fills, and of
+// the rule for cluster sizes. C entries for ctypes.
 #include <cmath>
 #include <vector>
 
@@ -59,3 +59,5 @@ extern "C" int tree_host_step(int n, int M, const double* src, double* dst) {
     }
   return bad ? 1 : 0;
 }
+
+extern "C" int tree_host_cluster(int n, int count, int slots, int most) { return tree_cluster(n, count, slots, most); }
