@@ -49,11 +49,25 @@ constexpr double kTreeGrowth = 2.26;
 // Level from which a unit is worked off breadth first: 5 takes 5.31 ms at N = 40 (levels too narrow
 // for a CTA), 7 takes 23.6 ms at N = 44 (its storage leaves the L2), 6 takes 4.7 and 22.0.
 constexpr int kTreeTop = 6;
-// Smallest scaled result that is kept. The tree's absolute error is about 2^-80 (against a
-// 113-bit evaluation), so 2^-28 leaves it at 2^-52 of the result. The subset sum it would be
-// handed back to is itself 2^-47 off at N = 32, 2^-42 at N = 40 and 2^-31 at N = 56, so the line
-// follows it down from N = 28 on: 2^-44 relative at N = 40, 2^-34 at N = 56.
-__device__ __forceinline__ int tree_min_exp(int n) { return n > 14 ? -28 - (4 * (n - 14)) / 3 : -28; }
+// Smallest scaled result that is kept: where the tree's absolute error is 2^-53 of it. The error is
+// a mean over the leaves: against a 113-bit evaluation, over matrices with loop weights of 0.2 to 2,
+// at most 2^-81.4 at N = 20, 2^-82.2 at 24, 2^-83.5 at 28 and 2^-84.0 at 32. (Configuration matrices
+// come out at 2^-20 for N = 40, 2^-27 for N = 50.)
+__device__ __forceinline__ int tree_min_exp(int n) { return n > 10 ? -28 - (n - 10) / 2 : -28; }
+
+// The scale of a vertex: d_j with lhaf(D A D) = det D lhaf(A). The edges alone ask for d^-2 = rho
+// (below) and for entries below 0.8; where the loop weights are large their vertices get a smaller
+// one, d_j |v_j| = sqrt(tau), such that sum d^2 |v|^2 <= kWeightSum: the weights enter g as exp of half
+// that sum spread over n pairs. Large weights and a full matrix together grow faster than each alone, so
+// d^-2 is raised by up to kWeightEdge as the sum approaches its limit. One scale for all vertices, as
+// the largest weight needs it, loses the smaller ones: of 152 matrices with weights of 0.3 to 2 a size (in and out
+// of phase, and random real ones) 35 were handed back to the subset sum at N = 20, 70 at 24, 105 at
+// 28; this way 0, 2 and 21. kWeightSum = 6.25 or 6.75: 1 or 4 at N = 24, 45 or 20 at N = 28.
+constexpr float kWeightSum = 6.5f, kWeightMax = 0.8f;
+constexpr float kWeightEdge = 0.75f, kWeightFree = 0.2f;
+// Weights beyond 2^32 times what the edges scale to one stay with the subset sum, whose value
+// test_handed_back_to_the_subset_sum (tests/test_gpu_tree.py) asks for there.
+constexpr float kWeightRange = 18446744073709551616.f;
 
 __device__ __forceinline__ void dd_two_prod(double a, double b, double& p, double& e) {
   p = __dmul_rn(a, b);
@@ -112,9 +126,10 @@ constexpr int kRootWarps = kRootThreads / 32;
 
 struct RootShared {
   float2 a[kMaxN * kMaxN];
+  float v2[kMaxN];          // |v_j|^2
+  short m[kMaxN], e[kMaxN];  // scale of index j: m / 16 2^e
   unsigned ea[kRootWarps], ev[kRootWarps];
-  float f[5][kRootWarps];
-  int m, e;
+  float f[3][kRootWarps];
 };
 
 __device__ __forceinline__ float warp_sum(float x) {
@@ -153,7 +168,7 @@ __device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState
     ev = max(ev, sh.ev[w]);
   }
   // entries and weights as floats below 2
-  float f2 = 0.f, am = 0.f, v2 = 0.f, vm = 0.f;
+  float f2 = 0.f, am = 0.f;
   for (int e = tid; e < N * N; e += kThreads) {
     const int r = e / N, c = e - r * N;
     const double2 z = tree_entry(P.in, r, c);
@@ -161,8 +176,7 @@ __device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState
     float2 w = make_float2(scaled_float(z.x, ex), scaled_float(z.y, ex));
     const float m2 = w.x * w.x + w.y * w.y;
     if (r == c) {
-      v2 += m2;
-      vm = fmaxf(vm, m2);
+      sh.v2[r] = m2;
       w = make_float2(0.f, 0.f);
     } else {
       f2 += m2;
@@ -188,66 +202,79 @@ __device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState
   }
   f2 = warp_sum(f2);
   g2 = warp_sum(g2);
-  v2 = warp_sum(v2);
   am = warp_max(am);
-  vm = warp_max(vm);
   if (lane == 0) {
     sh.f[0][warp] = f2;
     sh.f[1][warp] = g2;
-    sh.f[2][warp] = v2;
-    sh.f[3][warp] = am;
-    sh.f[4][warp] = vm;
+    sh.f[2][warp] = am;
   }
   __syncthreads();
-  if (tid == 0) {
-    f2 = g2 = v2 = am = vm = 0.f;
-    for (int w = 0; w < kWarps; ++w) {
-      f2 += sh.f[0][w];
-      g2 += sh.f[1][w];
-      v2 += sh.f[2][w];
-      am = fmaxf(am, sh.f[3][w]);
-      vm = fmaxf(vm, sh.f[4][w]);
+  if (warp == 0) {  // short code: a CTA runs it once and waits for its instructions
+    f2 = warp_sum(lane < kWarps ? sh.f[0][lane] : 0.f);
+    g2 = warp_sum(lane < kWarps ? sh.f[1][lane] : 0.f);
+    am = warp_max(lane < kWarps ? sh.f[2][lane] : 0.f);
+    // d^-2 of the edges alone, in units of 2^xa; |v|^2 is in units of 2^xv. Without edges the
+    // weights alone set the scales.
+    const int xv = 2 * ((int)ev - 1023);
+    int xa = (int)ea - 1023;
+    float da = fmaxf(f2 > 0.f ? sqrtf(__fdividef(g2, f2)) : 0.f, 1.25f * sqrtf(am));
+    if (ea == 0 || !(da > 0.f)) {
+      da = 1.f;
+      xa = ev ? xv - 60 : 0;
     }
-    // The loop weights enter g as exp of about |v|^2 / 2 spread over n pairs, hence |v|^2 / 8;
-    // |A_jk| and |v_j|^2 at most 0.8 keep A_jk + v_j v_k and 2 v_j v_k inside the format. den is
-    // in units of 2^top; a part that is far below the other does not count.
-    const int xa = (int)ea - 1023, xv = 2 * ((int)ev - 1023);
-    const float da = fmaxf(f2 > 0.f ? sqrtf(g2 / f2) : 0.f, 1.25f * sqrtf(am));
-    const float dv = fmaxf(v2 * 0.125f, 1.25f * vm);
-    int top = da > 0.f ? xa : xv;
-    if (dv > 0.f && xv > top) top = xv;
-    float den = fmaxf(da > 0.f && xa - top > -100 ? ldexpf(da, xa - top) : 0.f,
-                      dv > 0.f && xv - top > -100 ? ldexpf(dv, xv - top) : 0.f);
-    if (!(den > 0.f)) {
-      den = 1.f;
-      top = 0;
+    // d^2 |v|^2 of indices lane and lane + 32
+    const float m0 = lane < N ? sh.v2[lane] : 0.f, m1 = lane + 32 < N ? sh.v2[lane + 32] : 0.f;
+    const float unit = __fdividef(__int_as_float((min(max(xv - xa, -126), 126) + 127) << 23), da);
+    float w0 = m0 * unit, w1 = m1 * unit;
+    if (fmaxf(w0, w1) > kWeightRange) bad = 1;
+    const float full = warp_sum(fminf(w0, kWeightMax) + fminf(w1, kWeightMax)) * (1.f / kWeightSum);
+    const float edge = 1.f + kWeightEdge / (1.f - kWeightFree) * fmaxf(0.f, fminf(full, 1.f) - kWeightFree);
+    da *= edge;
+    w0 = __fdividef(w0, edge);
+    w1 = __fdividef(w1, edge);
+    float tau = kWeightMax;
+    if (full > 1.f && warp_sum(fminf(w0, tau) + fminf(w1, tau)) > kWeightSum) {
+      // the tau at which the sum of min(w, tau) is kWeightSum, from below
+      tau = __fdividef(kWeightSum, (float)N);
+#pragma unroll 1
+      for (int it = 0; it < 6; ++it) {
+        const float small = warp_sum((w0 <= tau ? w0 : 0.f) + (w1 <= tau ? w1 : 0.f));
+        const int big = __popc(__ballot_sync(0xffffffffu, w0 > tau)) + __popc(__ballot_sync(0xffffffffu, w1 > tau));
+        if (big) tau = fminf(__fdividef(kWeightSum - small, (float)big), kWeightMax);
+      }
     }
-    if (top & 1) {
-      den *= 2.f;
-      --top;
-    }
-    int ex;
-    // vertex scale 1 / sqrt(den 2^top), a little below, its mantissa cut to 5 bits: exact products
-    const float f = frexpf(rsqrtf(den) * 0.999999f, &ex);
-    sh.m = (int)(f * 32.f);
-    sh.e = ex - 1 - top / 2;  // scale = m / 16 * 2^e
-    if (!(sh.m >= 16 && sh.m <= 31) || sh.e > 900 || sh.e < -900) {
-      sh.m = 16;
-      sh.e = 0;
-      bad = 1;
+#pragma unroll 1
+    for (int j = lane; j < N; j += 32) {
+      const bool heavy = (j < 32 ? w0 : w1) > tau;
+      const float den = heavy ? __fdividef(j < 32 ? m0 : m1, tau) : da;
+      const int top = heavy ? xv : xa;
+      // 1 / sqrt(den 2^top), a little below, as m / 16 2^e with m of 5 bits: exact products
+      const int f = __float_as_int(rsqrtf((top & 1) ? 2.f * den : den) * 0.999999f);
+      const int e = (f >> 23) - 127 - (top >> 1);
+      if (e > 900 || e < -900) bad = 1;
+      sh.m[j] = (short)(16 + ((f >> 19) & 15));
+      sh.e[j] = (short)min(max(e, -900), 900);
     }
   }
   __syncthreads();
-  const int m = sh.m, e2 = sh.e;
-  if (tid == kThreads - 1) {  // 1 / scale^N: (16 / m)^N by squaring, exponents apart
-    double bh = 16.0 / m, bl = __fma_rn(-bh, (double)m, 16.0) / m, h = 1.0, l = 0.0;
-    for (int k = N; k > 0; k >>= 1) {
-      if (k & 1) dd_mul(h, l, bh, bl, h, l);
-      dd_mul(bh, bl, bh, bl, bh, bl);
+  if (warp == kWarps - 1) {  // 1 / det D: the product of the m / 16, and the exponents apart
+    double h = 1.0, l = 0.0;
+    int e = 0;
+    for (int j = lane; j < N; j += 32) {
+      h *= sh.m[j];
+      e += sh.e[j];
     }
-    S->fac_hi = h;
-    S->fac_lo = l;
-    S->exp2 = -kTreeFrac - (P.n >= 3 ? P.n - 3 : 0) - e2 * N + (P.Ne - N);
+    for (int d = 1; d < 4; d <<= 1) h *= __shfl_xor_sync(0xffffffffu, h, d);  // exact: 8 factors of 5 bits
+#pragma unroll 1
+    for (int d = 4; d < 32; d <<= 1)
+      dd_mul(h, l, __shfl_xor_sync(0xffffffffu, h, d), __shfl_xor_sync(0xffffffffu, l, d), h, l);
+    e = __reduce_add_sync(0xffffffffu, e);
+    if (lane == 0) {
+      const double r = __drcp_rn(h);
+      S->fac_hi = r;
+      S->fac_lo = __fma_rn(-r, l, __fma_rn(-r, h, 1.0)) * r;
+      S->exp2 = -kTreeFrac - (P.n >= 3 ? P.n - 3 : 0) - e + 4 * N + (P.Ne - N);
+    }
   }
   // root level: vertex 2 p is index p, vertex 2 p + 1 is index p + n; padding vertices have no
   // edges, loop weight one and scale one half
@@ -259,7 +286,7 @@ __device__ void tree_root(const TreeProblem& P, const TreeLevel& root, TreeState
     Fxc v{};
     if (r < N && c < N) {
       const double2 z = tree_entry(P.in, r, c);
-      const int mm = j == k ? m : m * m, ee = j == k ? e2 - 4 : 2 * e2 - 8;
+      const int mm = j == k ? sh.m[r] : sh.m[r] * sh.m[c], ee = j == k ? sh.e[r] - 4 : sh.e[r] + sh.e[c] - 8;
       to_fixed(z.x, mm, ee, v.rh, v.rm, v.rl, bad);
       to_fixed(z.y, mm, ee, v.ih, v.im, v.il, bad);
     } else if (j == k) {

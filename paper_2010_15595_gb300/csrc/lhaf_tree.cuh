@@ -32,11 +32,13 @@
 // operands from L1, against 0.17e12/s at best for triple-float (216 FP32 instructions) and
 // 0.15e12/s for FP64. (The integer multiply-add issues every 2 cycles when it repeats its
 // operands, 18.7e12/s, and every 4.4 in this code: its operand fetch is the limit.) Fixed point
-// needs a scale: the matrix is scaled by one factor such that its root-mean-fourth singular value
-// is about one, which keeps the coefficients of every matrix tried between 2^-10 and 2.5 (the
-// format holds |x| < 4, long levels a little less: fx_limit).
-// Overflow anywhere, or a result so small that the 2^-81 resolution could show, sets a flag and
-// the caller evaluates the problem by the subset sum instead.
+// needs a scale: each vertex gets one, such that the root-mean-fourth singular value of the matrix is
+// about one and no loop weight stands out (tree_root, lhaf_tree.cu). The coefficients of configuration
+// matrices then stay below 2.4 up to N = 32 and below 3.4 up to N = 50; the format holds |x| < 4,
+// long levels a little less (fx_limit). Overflow anywhere, or a result so small that the resolution could
+// show, sets a flag and the caller evaluates the problem by the subset sum instead: strongly graded
+// matrices, and from N = 26 on loop weights well above the entries (up to a seventh of them at N = 28, half at
+// N = 32, where weights of one phase and those above 1 come out too small).
 //
 // The code of one level is a function of (level, task number) that reads the level's nodes
 // and writes the next level's, so it compiles for the host as well and is checked there
