@@ -1,6 +1,8 @@
 """Launch-shape autotuner of the loop-hafnian kernels.
 
-Two kinds of entries, both timed through the C ABI on seeded synthetic inputs:
+Two kinds of entries, both timed through the C ABI on seeded synthetic inputs. They shape the
+launches of the subset sum, so the timed calls ask for sum |p_Z|, which only that evaluation
+gives (without it most sizes go to the elimination tree, which has no such entries):
 
 * single evaluations of size N (gbsh_lhaf*, per precision FP64 / triple-float): the cap on
   warps per CTA, the popcount-class ladder (coarse or fine steps of warps per CTA) and the
@@ -113,10 +115,10 @@ def tune_batch(n_max: int, precision: int = lib.PREC_FP64, candidates=CANDIDATES
         for w in candidates:
             try:
                 lib.set_batch_tuning(precision, n_max, w, warps_small=w0)
-                lib.lhaf_batch(mats, precision=precision)  # warm-up
+                lib.lhaf_batch(mats, precision=precision, return_abs_sum=True)  # warm-up
                 t0 = time.perf_counter()
                 for _ in range(reps):
-                    lib.lhaf_batch(mats, precision=precision)
+                    lib.lhaf_batch(mats, precision=precision, return_abs_sum=True)
                 times[(w0, w)] = (time.perf_counter() - t0) / reps
             except lib.GbshError:
                 continue
@@ -135,11 +137,11 @@ def tune_batch(n_max: int, precision: int = lib.PREC_FP64, candidates=CANDIDATES
 
 
 def _time_lhaf(A_dev, precision: int, reps: int) -> float:
-    lib.lhaf(A_dev, precision=precision)  # warm-up (also builds the plan's scratch)
+    lib.lhaf(A_dev, precision=precision, return_error=True)  # warm-up (also builds the plan's scratch)
     best = float("inf")
     for _ in range(reps):
         t0 = time.perf_counter()
-        lib.lhaf(A_dev, precision=precision)
+        lib.lhaf(A_dev, precision=precision, return_error=True)
         best = min(best, time.perf_counter() - t0)
     return best
 
