@@ -395,8 +395,9 @@ int gbsh_lhaf_ex(const gbsh_c128* A, int N, int lda, int precision, gbsh_c128* o
   if (!on_dev) {
     double2* dA = reinterpret_cast<double2*>(static_cast<char*>(ws) + in_off);
     if (host && type == cudaMemoryTypeUnregistered) {
-      // at most 50 kB; page-locked memory may still be written by what is on the stream, pageable
-      // memory is read at once either way
+      // At most 58 kB. What is on the stream may still write A (a host function, or a kernel where
+      // the device reaches pageable memory), which a copy on the stream waits for too.
+      GBSH_CUDA(cudaStreamSynchronize(st));
       double2* h = reinterpret_cast<double2*>(host + kHostInput);
       for (int r = 0; r < N; ++r) std::memcpy(h + (size_t)N * r, A + (size_t)lda * r, sizeof(double2) * N);
       GBSH_CUDA(cudaMemcpyAsync(dA, h, sizeof(double2) * N * N, cudaMemcpyHostToDevice, st));
