@@ -197,6 +197,22 @@ int tree_sync(gbsh::TreePlan* tp, const gbsh::BatchInput& in, void* ws, void* ho
   return GBSH_OK;
 }
 
+// Copies a host matrix (at most 58 kB) to the device through page-locked memory `h`. It is read at
+// once, but what the stream held before may still write it (a host function, or a kernel where the
+// device reaches pageable memory), which a copy from pageable memory waits for. So the caller asks
+// after the evaluation, when all that has run, whether the matrix is still what was read, and
+// starts again if not. (Asking for an idle stream or waiting for one beforehand takes 4 us of a
+// call's 333 at N = 32; comparing less than one.)
+cudaError_t stage_matrix(const gbsh_c128* A, int N, int lda, char* h, double2* dA, cudaStream_t st) {
+  for (int r = 0; r < N; ++r) std::memcpy(h + sizeof(double2) * N * r, A + (size_t)lda * r, sizeof(double2) * N);
+  return cudaMemcpyAsync(dA, h, sizeof(double2) * N * N, cudaMemcpyHostToDevice, st);
+}
+bool staged_matrix(const gbsh_c128* A, int N, int lda, const char* h) {
+  for (int r = 0; r < N; ++r)
+    if (std::memcmp(h + sizeof(double2) * N * r, A + (size_t)lda * r, sizeof(double2) * N) != 0) return false;
+  return true;
+}
+
 // ---------------------------------------------------------------- batched evaluation
 using gbsh::BatchLayout;
 using gbsh::batch_layout;
@@ -392,15 +408,12 @@ int gbsh_lhaf_ex(const gbsh_c128* A, int N, int lda, int precision, gbsh_c128* o
   char* host = tree ? scratch_host(s) : nullptr;
   const double2* base = reinterpret_cast<const double2*>(A);
   int ld = lda;
+  bool staged = false;
   if (!on_dev) {
     double2* dA = reinterpret_cast<double2*>(static_cast<char*>(ws) + in_off);
-    if (host && type == cudaMemoryTypeUnregistered) {
-      // At most 58 kB. What is on the stream may still write A (a host function, or a kernel where
-      // the device reaches pageable memory), which a copy on the stream waits for too.
-      GBSH_CUDA(cudaStreamSynchronize(st));
-      double2* h = reinterpret_cast<double2*>(host + kHostInput);
-      for (int r = 0; r < N; ++r) std::memcpy(h + (size_t)N * r, A + (size_t)lda * r, sizeof(double2) * N);
-      GBSH_CUDA(cudaMemcpyAsync(dA, h, sizeof(double2) * N * N, cudaMemcpyHostToDevice, st));
+    staged = host && type == cudaMemoryTypeUnregistered;
+    if (staged) {
+      GBSH_CUDA(stage_matrix(A, N, lda, host + kHostInput, dA, st));
     } else {
       GBSH_CUDA(cudaMemcpy2DAsync(dA, sizeof(double2) * N, A, sizeof(double2) * lda,
                                   sizeof(double2) * N, N, cudaMemcpyHostToDevice, st));
@@ -410,7 +423,12 @@ int gbsh_lhaf_ex(const gbsh_c128* A, int N, int lda, int precision, gbsh_c128* o
   }
   if (tree) {
     bool done = false;
-    rc = tree_sync(&tp, gbsh::BatchInput{base, nullptr, nullptr, ld, N}, ws, host, st, out, &done);
+    const gbsh::BatchInput in{base, nullptr, nullptr, ld, N};
+    rc = tree_sync(&tp, in, ws, host, st, out, &done);
+    if (rc == GBSH_OK && staged && !staged_matrix(A, N, lda, host + kHostInput)) {
+      GBSH_CUDA(stage_matrix(A, N, lda, host + kHostInput, const_cast<double2*>(base), st));
+      rc = tree_sync(&tp, in, ws, host, st, out, &done);
+    }
     if (rc != GBSH_OK || done) return rc;
   }
   double asum = 0.0;
