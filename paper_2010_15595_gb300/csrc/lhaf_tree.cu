@@ -40,6 +40,7 @@ constexpr int kTreeCtasPerSm = 5;
 // against 108: their levels are wider than 16 CTAs. 128 unrelated matrices of up to 16 indices
 // take 195 us with this line at 8 or 9, 255 at 7.
 constexpr int kTreeSmallMax = 8;
+static_assert(kTreeSmallMax <= kFxLimitFree, "the limit of small problems is a constant");
 // Units (tasks of one CTA) that a launch aims at, per CTA that runs at a time, shared out by work:
 // a tree's work grows 2.26-fold with an index pair (n = 16 to 22). 512 patterns of up to 30
 // photons take 7.6 ms with 2, 7.06 with 4, 6.75 with 8, 6.63 with 16, and 10.0 with 2 shared
@@ -559,7 +560,7 @@ tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int fi
   for (int p = first + id; p < first + count; p += clusters) {
     const TreeProblem P = kOne ? one : table[p];
     TreeState* S = state + p;
-    if (tid < P.n) phase[tid] = tree_whole_phase(base, P.n, tid);
+    if (tid < P.n) phase[tid] = tree_whole_phase<true>(base, P.n, tid);
     if (tid == P.n) s_bad = 0;
     if (rank == 0) tree_root<kRootThreads>(P, tree_level(base, P.n, P.n, 1), S, sh.root);
     __syncthreads();
@@ -577,11 +578,12 @@ tree_small_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int fi
       if (pieces <= 3 * stride) {
         for (int q = t0; (q & ~31) < pieces; q += stride) {
           if (q != t0) J = tree_piece_job(s, q, t);
+          J.lim = kFxLimit;
           if (tree_piece_task(J, t, q & 3, z, bad)) sh.sum.add(z, __popc((unsigned)J.node) & 1);
         }
       } else {
         for (int q = t0; q < s.tasks; q += stride)
-          if (tree_task(s, 0, q, JobSlot<kRootThreads>{slots}, x, z, bad)) sh.sum.add(z, __popc((unsigned)x) & 1);
+          if (tree_task<true>(s, 0, q, JobSlot<kRootThreads>{slots}, x, z, bad)) sh.sum.add(z, __popc((unsigned)x) & 1);
       }
       if (i == P.n - 1) {
         if (bad) atomicOr(&s_bad, 1u);

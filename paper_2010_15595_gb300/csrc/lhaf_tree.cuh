@@ -164,9 +164,11 @@ GBSH_HD Fxc fx_norm(const FxSum& s, unsigned& over) {
 // stays below the 1020 that fx_norm1 needs if the numbers are below sqrt(255 / L): 4 up to 15
 // coefficients (N = 34), then less, 3.57 at N = 44 (where a configuration matrix was seen to reach
 // 3.31), 3.02 at N = 60. Level 2's numbers enter single products and may be as large as 4 at any length.
+constexpr int kFxLimitFree = 15;  // coefficients up to which it is 4
+constexpr int kFxLimit = (4 << (kTreeFrac - 2 * kLimbBits)) - 1;
 GBSH_HD int fx_limit(int L) {
   constexpr int kOne = 1 << (kTreeFrac - 2 * kLimbBits);
-  if (L <= 15) return 4 * kOne - 1;
+  if (L <= kFxLimitFree) return kFxLimit;
 #ifdef __CUDA_ARCH__
   return (int)(sqrtf(255.0f / (float)L) * (float)kOne) - 64;  // 64: roundings of the root
 #else
@@ -339,13 +341,15 @@ struct TreePhase {
 
 // A task makes coefficients in twos: a tile near the top and its mirror tile near the bottom of
 // an item's triangle of products, so that all tasks of a phase cost the same.
+// kShort: n is at most kFxLimitFree, and the limit is known without the root's code.
+template <bool kShort = false>
 GBSH_HD void tree_ready(TreePhase& s) {
   const int L = s.n - s.M + 1, g = s.M < s.n ? s.par.q : 0;
   const int per = s.kind == kTreeStep ? tree_polys(s.M - 1) : (s.kind == kTreeLast1 ? 6 : 4);
   s.nmain = s.src.q * (s.kind == kTreeStep ? per + 1 : per);
   s.items = s.nmain + (s.kind == kTreeLast2 ? 0 : g);
   s.tasks = ((L + 1) / 2 + 1) / 2 * s.items;
-  s.lim = fx_limit(s.kind == kTreeStep && s.M > 3 ? L + 1 : 0);
+  s.lim = kShort ? kFxLimit : fx_limit(s.kind == kTreeStep && s.M > 3 ? L + 1 : 0);
   s.inv_items = 1.0f / (float)s.items;
   s.inv_node = 1.0f / (float)per;
 }
@@ -577,8 +581,9 @@ GBSH_HD TreeJob tree_get(const Slot& m, const char* fb, int lim) {
 }
 
 // Runs one task of walk `walk`. In phase last2 returns true with a part of node `node`'s term in
-// z (sums of limbs, carries not propagated). bad: 0, or 1 once a number left the range.
-template <class Slot>
+// z (sums of limbs, carries not propagated). bad: 0, or 1 once a number left the range. kShort: n is
+// at most kFxLimitFree, and the limit is known without the phase.
+template <bool kShort = false, class Slot>
 GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& slot, int& node, Fxc& z,
                        unsigned& bad) {
   int tile = tree_div(task, s.items, s.inv_items);
@@ -625,7 +630,7 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
         const Fxc v = fx_norm(sum, over);
         sum = sum1;
         if (t < 0) continue;
-        const TreeJob J = tree_get(slot, fb, s.lim);
+        const TreeJob J = tree_get(slot, fb, kShort ? kFxLimit : s.lim);
         if (J.end == kDot) {
           FxAcc dot = fx_acc_zero();
           fx_mac(dot, v, fx_load(fb + J.old + (ptrdiff_t)(J.last - t) * J.so));
@@ -647,6 +652,7 @@ GBSH_HD bool tree_task(const TreePhase& s, unsigned walk, int task, const Slot& 
 // ------------------------------------------------------------------ cutting the tree
 // Phase i of n of the whole tree breadth first; its levels n, n - 1, ... follow each other from
 // `base`.
+template <bool kShort = false>
 GBSH_HD TreePhase tree_whole_phase(char* base, int n, int i) {
   TreePhase s;
   const int M = n - i > 2 ? n - i : 2;
@@ -660,7 +666,7 @@ GBSH_HD TreePhase tree_whole_phase(char* base, int n, int i) {
   s.single = i == 0 && n > 2;
   s.psign = M == n - 1 ? 1 : 0;
   s.src_bit = s.par_bit = -1;
-  tree_ready(s);
+  tree_ready<kShort>(s);
   return s;
 }
 
