@@ -47,6 +47,11 @@ static_assert(kTreeSmallMax <= kFxLimitFree, "the limit of small problems is a c
 // out evenly; the storage for the levels above the units grows with it.
 constexpr double kTreeUnits = 8;
 constexpr double kTreeGrowth = 2.26;
+// Levels above the units at most, which bounds their storage: 2048 units, fewer than kTreeUnits asks
+// for from one problem of N = 27 on. N = 50 takes 212 ms and 1.8 GB with 12, 218 and 1.8 with 11, 211 and 2.0 with
+// 13; N = 56 2.10 s, 2.21 and 2.12. 13 suits N = 40 (4.21 ms, 4.70 with 12) and 48 (94 ms, 100), but takes
+// 375 us instead of 319 at N = 32 and 1.05 ms instead of 1.02 at N = 36.
+constexpr int kTreeDepth = 12;
 // Level from which a unit is worked off breadth first: 5 takes 5.31 ms at N = 40 (levels too narrow
 // for a CTA), 7 takes 23.6 ms at N = 44 (its storage leaves the L2), 6 takes 4.7 and 22.0.
 constexpr int kTreeTop = 6;
@@ -468,9 +473,10 @@ struct LimbSums {
 // The units of all large problems, claimed from a counter by one resident wave of CTAs: nearly all
 // of a large evaluation. A unit's levels live in the CTA's own scratch (walked depth first, two
 // nodes a level, so that the scratch of all CTAs stays in the L2) and its tasks are independent
-// within a phase. Bound by the convolutions' multiply-adds (70 %, see fx_conv2) and the latency of
-// their loads (43 % hit L1, and a warp waits for one during 27 % of its time). N = 40: 4.65 ms, 0.22e12 complex
-// multiply-adds/s (184 ms for the subset sum); N = 44: 21.6 ms (919).
+// within a phase. Bound by the convolutions' multiply-adds (their pipe is busy 69 % of the time, see
+// fx_conv2), and the latency of their loads (4.4 warps a scheduler; 50 % hit L1, and a
+// warp waits for one during 15 % of its time). N = 40: 4.70 ms, 0.21e12 complex
+// multiply-adds/s (184 ms for the subset sum); N = 44: 20.8 ms (919).
 template <bool kOne>
 __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm)
 tree_kernel(const TreeProblem* __restrict__ table, TreeProblem one, int count, unsigned total_units,
@@ -709,7 +715,7 @@ cudaError_t tree_plan(const int* Ns, int count, size_t base_off, TreePlan* plan)
     if (q >= T.nbig) continue;
     P.m1 = n - 1;
     const double want = kTreeUnits * slots * std::pow(kTreeGrowth, n) / work;
-    while (P.m1 > 2 && tree_width(P.m1, n) < want && n - P.m1 < (n > 24 ? 11 : 12)) --P.m1;
+    while (P.m1 > 2 && tree_width(P.m1, n) < want && n - P.m1 < kTreeDepth) --P.m1;
     P.top = std::min(kTreeTop, P.m1);
     P.units = (unsigned)tree_width(P.m1, n);
     base += P.units;
