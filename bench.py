@@ -570,8 +570,9 @@ def run_batch_workload(lib, workloads, workmodel, dev, stream, count=4096):
     """Batched workload: 4096 loop hafnians of uneven size (N uniform on even 10..30) from
     one M=100-mode state (r=0.7, Haar U, gamma ~ CN(0, 0.1^2)), up to 3 photons per mode,
     through gbsh_gbs_prob_batch (device B and gamma), in FP64, GBSH_PREC_TF and complex FP32.
-    Errors: every FP64 and FP32 result against the GBSH_PREC_TF result of the same problem
-    (which the tests hold within 1e-9 of the oracle)."""
+    Errors: every FP32 result, and the FP64 ones above N = 24 (up to there FP64 and GBSH_PREC_TF are
+    the same evaluation), against the GBSH_PREC_TF result of the same problem (which the tests
+    hold within 1e-9 of the oracle)."""
     import numpy as np
     import torch
     B, gamma = workloads.batch_state()
@@ -605,8 +606,9 @@ def run_batch_workload(lib, workloads, workmodel, dev, stream, count=4096):
                              "unit": "T integer multiply-adds/s",
                              "frac": ach / workmodel.IMAD_PEAK_DERIVED_T}
     for name in ("fp64", "c32"):
-        err = np.abs(out[name] - out["tf"]) / np.abs(out["tf"])
-        res[name]["rel_err_vs_tf"] = {"median": float(np.median(err)),
+        some = Ns > 24 if name == "fp64" else Ns > 0
+        err = np.abs(out[name] - out["tf"])[some] / np.abs(out["tf"])[some]
+        res[name]["rel_err_vs_tf"] = {"problems": int(some.sum()), "median": float(np.median(err)),
                                       "p99": float(np.quantile(err, 0.99)), "max": float(err.max())}
     res["c32"]["enabled_by_mixed_mode_for_N_le"] = lib.C32_MAX_N
     return res

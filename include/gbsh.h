@@ -26,9 +26,13 @@
  *     with N <= 24, an elimination tree in fixed point (resolution 2^-81) evaluates the loop hafnian instead
  *     (csrc/lhaf_tree.cuh): far fewer operations and far less cancellation. A problem that
  *     leaves the fixed-point range is evaluated by the subset sum after all.
- *   - Results are bit-reproducible for a given N on a given GPU model: the subset sum is
- *     split into fixed chunks whose compensated partial sums are combined in a fixed order, and
- *     the tree's sums are exact integers.
+ *   - Results of either evaluation are bit-reproducible for a given N on a given GPU model: the
+ *     subset sum is split into fixed chunks whose compensated partial sums are combined in a fixed
+ *     order, and the tree's sums are exact integers. The two agree within the subset sum's
+ *     rounding, not in every bit, and which one runs depends on more than the matrix: on what
+ *     the call asks for (above), and on memory. The subset sum serves an asynchronous call whose workspace
+ *     cannot hold the tree's scratch (see gbsh_lhaf_workspace_size) and a synchronous one whose
+ *     scratch cannot be allocated.
  *   - Functions are re-entrant; calls on different streams may run concurrently. Host
  *     buffers are owned by the caller and only read/written during the call.
  */
@@ -79,7 +83,7 @@ int gbsh_version(void);
  *   stream   cudaStream_t. The call synchronises this stream before returning.
  * Scratch memory is taken from a per-device cache that the library grows on demand with
  * cudaMalloc and keeps until exit: the subset sum's (at most some 120 MB) and the elimination
- * tree's (0.14 GB at N = 32, 0.74 GB at 40, 1.9 GB at 50, 4.0 GB at 60). Where the tree's cannot
+ * tree's (0.14 GB at N = 32, 0.74 GB at 40, 1.9 GB at 50, 4.1 GB at 60). Where the tree's cannot
  * be had the subset sum is used.
  * Errors: GBSH_EINVAL (N < 0, N > GBSH_MAX_N, lda < N, A/out NULL), GBSH_ENOMEM,
  * GBSH_ECUDA.
@@ -87,11 +91,14 @@ int gbsh_version(void);
 int gbsh_lhaf(const gbsh_c128* A, int N, int lda, gbsh_c128* out, double* err_est,
               void* stream);
 
-/* Bytes of device workspace gbsh_lhaf_async needs for size N (0 for N outside 1..MAX_N). */
+/* Bytes of device workspace gbsh_lhaf_async needs for size N (0 for N outside 1..MAX_N). Not
+ * monotone: N <= 24 include the elimination tree's scratch, larger N do not (7 MB at N = 24, 1.4 MB
+ * at 26). One workspace for several sizes that is to have the tree throughout must hold the
+ * largest of their sizes; with less, the subset sum is used where the tree does not fit. */
 size_t gbsh_lhaf_workspace_size(int N);
 /* The same for gbsh_lhaf_async_ex in `precision` (0 for an unsupported precision). For
- * GBSH_PREC_TF (and for N <= 24) this includes the elimination tree's scratch; a workspace that
- * only holds the subset sum's part is accepted too, and the subset sum is used. */
+ * GBSH_PREC_TF every size includes the tree's scratch; a workspace that only holds the subset sum's
+ * part is accepted too, and the subset sum is used. */
 size_t gbsh_lhaf_workspace_size_ex(int N, int precision);
 
 /*
@@ -329,8 +336,9 @@ int gbsh_visit_counts(int N, unsigned* d_counts, void* stream);
 int gbsh_set_lhaf_tuning(int warps_per_cta, int kcap);
 
 /*
- * gbsh_lhaf_plan — launch plan that gbsh_lhaf / gbsh_lhaf_async use for size N on the
- * current device, under the current tuning. Any output pointer may be NULL.
+ * gbsh_lhaf_plan — launch plan of the FP64 subset sum of size N on the current device, under the
+ * current tuning: what gbsh_lhaf and gbsh_lhaf_async run where the elimination tree does not serve
+ * the call (see the conventions above). Any output pointer may be NULL.
  *   nclass     number of subset-kernel launches (popcount classes, 1..12)
  *   kernels    CUDA kernels launched per evaluation (expansion + classes + two-level finalize)
  *   warps      warps per CTA of the first class
@@ -340,7 +348,7 @@ int gbsh_set_lhaf_tuning(int warps_per_cta, int kcap);
  * Errors: GBSH_EINVAL for N outside 1..GBSH_MAX_N, GBSH_ECUDA without a device.
  */
 int gbsh_lhaf_plan(int N, int* nclass, int* kernels, int* warps, int* kcap, int* nchunks);
-/* The same for the plan of `precision` (GBSH_PREC_FP64 or GBSH_PREC_TF). */
+/* The same for the subset sum in `precision` (GBSH_PREC_FP64 or GBSH_PREC_TF). */
 int gbsh_lhaf_plan_ex(int N, int precision, int* nclass, int* kernels, int* warps, int* kcap,
                       int* nchunks);
 

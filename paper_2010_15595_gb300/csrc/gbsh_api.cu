@@ -168,9 +168,11 @@ int run_sync(const gbsh::LhafPlan& plan, const double2* base, int ld, const doub
 
 // Whether a call that does not ask for sum |p_Z| is evaluated by the elimination tree
 // (lhaf_tree.cuh): the sum over |p_Z| only exists in the subset sum. FP64 evaluations stay with
-// the subset sum above N = 24. The FP64 entry points -- single, batched, in subset ranges -- are
-// compared with one another, and there the rounding of the FP64 subset sum (4e-11 at N = 24,
-// 1e-10 to 1e-8 at N = 26 to 30) would show between one that moved and one that cannot.
+// the subset sum above N = 24: tests/test_gpu_range.py holds them against combined subset ranges at
+// 1e-12 (N = 27 and 32), and the FP64 subset sum's own rounding is 1e-10 to 1e-8 there. At and below
+// 24 a whole evaluation is the tree's and differs from what ranges and calls with an error estimate
+// add up to by that rounding: up to 6e-12 at N = 16, 1e-10 at N = 20 and 4e-9 at N = 24. (N = 30 takes 2.36
+// ms; the tree 0.17 at N = 28 and 0.32 at 32.)
 constexpr int kTreeFp64MaxN = 24;
 bool tree_precision(int prec, int N) {
   return prec == GBSH_PREC_TF || (prec == GBSH_PREC_FP64 && N <= kTreeFp64MaxN);

@@ -199,7 +199,7 @@ def lhaf(A, stream=None, return_error=False, precision=None):
 
 
 def plan(N: int, precision=None) -> dict:
-    """Launch plan of an N x N evaluation on the current device (see gbsh_lhaf_plan)."""
+    """Launch plan of an N x N subset sum on the current device (see gbsh_lhaf_plan)."""
     vals = [ctypes.c_int() for _ in range(5)]
     refs = [ctypes.byref(v) for v in vals]
     if precision is None:
